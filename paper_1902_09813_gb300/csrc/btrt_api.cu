@@ -367,6 +367,24 @@ void btrt::fill_params(btrt_lattice L, SweepParams<Real> &p, int64_t n, bool fir
         q.k6x3k = (Real)(k0 / 4.0);
         q.a2x3 = (Real)(3.0 * c.a2);
     }
+    if constexpr (std::is_same<Real, double>::value) {
+        // the same constants for the integer collision; where one does not fit (or is
+        // not finite), the kernels keep the FP64 form
+        const FoldConsts<double> &q = p.lin;
+        const double dk = L->k2 - c.k0;
+        const double v[10] = {-q.Qxx, -q.Qxy, -q.Qyy, q.Pgx, q.Pgy, -q.gx, -q.gy, dk, dk, q.om};
+        const int div[10] = {6, 6, 6, 6, 6, 6, 6, 18, 4, 2};
+        FxConst k[10];
+        bool ok = true;
+        for (int i = 0; i < 10; ++i) {
+            const bool fits = std::fabs(v[i]) < 0.4999 * div[i];
+            k[i] = fx_const(fits ? v[i] : 0.0, div[i]);
+            ok = ok && fits;
+        }
+        ok = ok && fx_flux_fits(k[0], k[1], k[3], k[5]) && fx_flux_fits(k[1], k[2], k[4], k[6]);
+        p.fx = FxFold{k[0], k[1], k[2], k[3], k[4], k[5], k[6], k[7], k[8], k[9],
+                      (std::fabs(q.om) < 0.9998 ? kFxOkGeneral : 0) | (ok ? kFxOkLinear : 0), 0};
+    }
     // the reference value of kShiftRef storage (zero otherwise)
     p.phi_ref = shift_of(g) == kShiftRef ? (Real)g.phi_ref : (Real)0.0;
     // stochastic rounding: the seed of step index n (the same in every kernel form)

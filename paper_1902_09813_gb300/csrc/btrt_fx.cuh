@@ -1,0 +1,303 @@
+// btrt_fx.cuh -- the FP64 collision in 64-bit block fixed point.
+//
+// GB300 issues fewer than two FP64 operations per SM and clock (0.527 T op/s
+// measured), so a collision of 50 FP64 operations takes 29 clocks per node while
+// nine tenths of the issue slots stay empty; HBM would allow one node per 7 clocks.
+// The collision of Eq. 6 is a linear map of the nine populations (plus a few
+// per-node terms), so it can run on the integer pipes instead: the populations of
+// one node are brought to one common exponent E (the largest among them), as 64-bit
+// integers in units of 2^(E - 58), their moments are exact integer sums, products
+// with the collision's constants are 64 x 64-bit products rounded to a unit, and
+// each result is rounded once to FP64 on its way out.
+//
+// Precision: the largest population has its 53 bits in the integer with five to
+// spare, so every intermediate carries an error of about one unit, 2^-58 of the
+// largest population, where FP64 arithmetic rounds each intermediate of that size
+// to 2^-53.  The four-times-smaller axis populations and the sixteen-times-smaller
+// diagonal ones keep errors at or below those of the FP64 form; their sum is exact
+// (r_0 is formed as the total minus the other eight).
+// Range: exponents 64 .. 2040 (about 1e-289 .. 1e306); below it a result is the
+// nearest multiple of 2^-1017, above it (and for infinities and NaN) the node takes
+// the FP64 form (collide_f64_slow).
+#pragma once
+
+#include <math.h>
+#include <stdint.h>
+#include <string.h>
+
+#ifdef __CUDACC__
+#define BTRT_HD __host__ __device__ __forceinline__
+#else
+#define BTRT_HD inline
+#endif
+
+namespace btrt {
+
+using fx = long long;
+
+constexpr unsigned int kFxExpMin = 64u << 20, kFxExpMax = 2040u << 20, kFxExpMask = 0x7ff00000u;
+
+// A constant C as (hi 2^32 + lo) = C 2^64, lo signed; |C| < 1/2.
+struct FxConst {
+    int hi, lo;
+};
+// v / div to the nearest unit: the integer division adds no rounding of its own to v's.
+inline FxConst fx_const(double v, int div) {
+    int e;
+    const __int128 m = (__int128)(long long)ldexp(frexp(v, &e), 53);   // v = m 2^(e - 53)
+    const int sh = 49 - e;                                             // (m 2^60 / div) 2^(e - 49) = v 2^64 / div
+    const __int128 q = m * ((__int128)1 << 60) / div;
+    const long long c = sh < 120 ? (long long)((q + ((__int128)1 << (sh - 1))) >> sh) : 0;
+    FxConst k;
+    k.lo = (int)(unsigned int)(unsigned long long)c;
+    k.hi = (int)((c - (long long)k.lo) >> 32);
+    return k;
+}
+
+BTRT_HD unsigned long long fx_bits(double v) {
+#ifdef __CUDA_ARCH__
+    return (unsigned long long)__double_as_longlong(v);
+#else
+    unsigned long long b;
+    memcpy(&b, &v, 8);
+    return b;
+#endif
+}
+BTRT_HD double fx_double(unsigned long long b) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double v;
+    memcpy(&v, &b, 8);
+    return v;
+#endif
+}
+// Exponent field of v, in place in the high word.
+BTRT_HD unsigned int fx_exp(double v) { return (unsigned int)(fx_bits(v) >> 32) & kFxExpMask; }
+
+// v in units of 2^(E - 58) (E = em >> 20, biased as in FP64), truncated toward
+// zero: the mantissa with its hidden bit at the top of the word, shifted down by
+// E + 5 - e.  Shifts of 64 and more give 0 (also for zeros and subnormals, whose
+// hidden bit is not there: E >= 64 shifts them out).  e <= E + 4.
+BTRT_HD fx fx_from(double v, unsigned int em) {
+    const unsigned long long b = fx_bits(v);
+    const unsigned int sh = (em + (5u << 20) - ((unsigned int)(b >> 32) & kFxExpMask)) >> 20;
+    unsigned long long m = (b << 11) | 0x8000000000000000ull;
+#ifdef __CUDA_ARCH__
+    asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(sh));   // PTX clamps the amount at 64
+#else
+    m = sh < 64 ? m >> sh : 0;
+#endif
+    const fx s = (fx)b >> 63;
+    return ((fx)m ^ s) - s;
+}
+
+// The FP64 value nearest to v 2^(E - 58) (ties away from zero).
+BTRT_HD double fx_to(fx v, unsigned int em) {
+    const fx s = v >> 63;
+    const unsigned long long a = (unsigned long long)((v ^ s) - s);
+    unsigned int hi = (unsigned int)(a >> 32), lo = (unsigned int)a, up = em + (4u << 20);
+    if (hi == 0) {
+        hi = lo;
+        lo = 0;
+        up -= 32u << 20;
+    }
+#ifdef __CUDA_ARCH__
+    const unsigned int lz = (unsigned int)__clz((int)hi);
+    const unsigned int mh = __funnelshift_l(lo, hi, lz), ml = lo << (lz & 31);
+#else
+    const unsigned int lz = hi ? (unsigned int)__builtin_clz(hi) : 32u;
+    const unsigned long long n = hi ? (((unsigned long long)hi << 32) | lo) << lz : 0ull;
+    const unsigned int mh = (unsigned int)(n >> 32), ml = (unsigned int)n;
+#endif
+    // mantissa with its hidden bit at bit 52, rounded; the hidden bit adds one to the exponent field
+    unsigned long long r = ((((unsigned long long)mh << 32) | ml) >> 11) + ((ml >> 10) & 1u);
+    r += (unsigned long long)(up - (lz << 20)) << 32;
+    r |= (unsigned long long)s & 0x8000000000000000ull;
+    return fx_double((int)mh < 0 ? r : 0ull);
+}
+
+// The same with two FP64 additions (ties to even): the words of v enter the
+// mantissas of 2^84 and 2^52, the constants leave again, and only the second
+// addition rounds.  The FP64 adder is otherwise idle here, but ten conversions
+// would make it the bound.
+BTRT_HD double fx_to_add(fx v, unsigned int em) {
+    const unsigned long long u = (unsigned long long)v;
+    const double b = fx_double(0x4530000000000000ull | ((u >> 32) ^ 0x80000000ull));
+    const double a = fx_double(0x4330000000000000ull | (u & 0xffffffffull));
+    const double r = (b - 19342822341709703277445120.0) + a;   // 2^84 + 2^63 + 2^52
+    const unsigned long long rb = fx_bits(r);
+    const unsigned int rh = (unsigned int)(rb >> 32);
+    return fx_double((unsigned long long)(rh ? rh + em - (1081u << 20) : 0u) << 32 | (rb & 0xffffffffull));
+}
+
+// x as h 2^32 + l with l signed, for the products below.
+struct FxArg {
+    int h, l;
+};
+BTRT_HD FxArg fx_arg(fx x) {
+    FxArg a;
+    a.l = (int)(unsigned int)(unsigned long long)x;
+    a.h = (int)(x >> 32) + (int)((unsigned int)a.l >> 31);
+    return a;
+}
+
+// Sum of products C_k x_k, |C_k| < 1/2: p counts units, t 2^-32 units (the products
+// of the two low words, at most a quarter of a unit per term, are left out).  t
+// starts at half a unit of the result, which rounds it.  The host checks that t
+// stays in range for the constants it hands out (fx_flux_fits).
+struct FxSum {
+    fx p, t;
+};
+BTRT_HD FxSum fx_sum() {
+    FxSum s;
+    s.p = 0;
+    s.t = 1ll << 31;
+    return s;
+}
+BTRT_HD void fx_add(FxSum &s, const FxArg &x, const FxConst &c) {
+    s.t += (fx)x.h * c.lo;
+    s.t += (fx)x.l * c.hi;
+    s.p += (fx)x.h * c.hi;
+}
+BTRT_HD fx fx_value(const FxSum &s) { return s.p + (fx)(int)(s.t >> 32); }
+BTRT_HD fx fx_mul(const FxArg &x, const FxConst &c) {
+    const fx t = (1ll << 31) + (fx)x.h * c.lo + (fx)x.l * c.hi;
+    return (fx)x.h * c.hi + (fx)(int)(t >> 32);
+}
+// Whether the sum qx jx + qy jy + cp phi + cg phi^{n-1} keeps t below 2^63 for every
+// node the integer path takes: populations below 2^59 units (high words below 2^27;
+// each enters the first three products with the coefficient ex qx + ey qy + cp),
+// phi^{n-1} below 2^62.
+inline bool fx_flux_fits(const FxConst &qx, const FxConst &qy, const FxConst &cp, const FxConst &cg) {
+    const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+    auto mag = [](double v) { return v < 0 ? -v : v; };
+    double t = 17179869184.0 + 1073741824.0 * mag(cg.lo);
+    for (int i = 0; i < 9; ++i) t += 134217728.0 * mag((double)ex[i] * qx.lo + (double)ey[i] * qy.lo + cp.lo);
+    t += 2147483648.0 * (mag(qx.hi) + mag(qy.hi) + mag(cp.hi) + mag(cg.hi) + 4.0);
+    return t < 9223372036854775808.0;
+}
+
+// x / 9, rounded to a unit.
+BTRT_HD fx fx_ninth(fx x) {
+    const FxConst c = {0x1c71c71c, 0x71c71c72};   // 2^64 / 9
+    return fx_mul(fx_arg(x), c);
+}
+
+// The constant-coefficient collision's constants (see collide_fold for the scheme
+// and the names): V/6 takes -(K1 - k0 I)/6 on the first moments, (K1 u^ + g)/6 on
+// phi and -g/6 on phi^{n-1}, g = (I - K1/2) u^; the second-order block takes
+// (k2 - k0)/18 on (3/2) sigma and (k2 - k0)/4 on delta and Pi_xy; om2 = (1 - k0)/2.
+struct FxFold {
+    FxConst Qxx, Qxy, Qyy, Px, Py, gx, gy, d18, d4, om2;
+    int ok;          // kFxOk* bits; a form whose bit is not set takes the FP64 collision
+    int pad;
+};
+enum { kFxOkGeneral = 1, kFxOkLinear = 2 };   // om2 fits; all of the constants fit
+
+// Populations after the collision from the node's integer moments: a = k0 phi +
+// source, z the term of C(phi) != phi, X, Y = V/6, ks = (k2 - k0) sigma / 12, and the
+// two anisotropic second-order terms t1 = (k2 - k0) delta / 4, t5 = (k2 - k0) Pi_xy / 4.
+BTRT_HD void fx_expand(fx a, fx z, fx X, fx Y, fx ks, fx t1, fx t5, fx (&r)[9]) {
+    const fx b = fx_ninth(a);
+    const fx zk = z - ks;
+    const fx T1 = b + zk, T5 = (b >> 2) + zk;
+    r[0] = a - 4 * (T1 + T5);           // the other eight sum to 4 (T1 + T5)
+    const fx A1 = T1 - t1, A2 = T1 + t1;
+    r[1] = A1 + 2 * X;
+    r[3] = A1 - 2 * X;
+    r[2] = A2 + 2 * Y;
+    r[4] = A2 - 2 * Y;
+    const fx P = T5 - t5, M = T5 + t5;
+    const fx Vp = (X + Y) >> 1, Vm = (X - Y) >> 1;
+    r[5] = P + Vp;
+    r[7] = P - Vp;
+    r[6] = M - Vm;
+    r[8] = M + Vm;
+}
+
+// Integer moments of a node.
+struct FxMoments {
+    fx phi, jx, jy, pxy, del, s32;   // s32 = (3/2) sigma = (a13 + a24)/2 + 2 (diagonals) - d0
+};
+BTRT_HD FxMoments fx_moments(const fx (&D)[9]) {
+    FxMoments m;
+    const fx a13 = D[1] + D[3], a24 = D[2] + D[4];
+    const fx s57 = D[5] + D[7], s68 = D[6] + D[8];
+    const fx d57 = D[5] - D[7], d68 = D[6] - D[8];
+    const fx sd = s57 + s68, a1324 = a13 + a24;
+    m.phi = D[0] + sd + a1324;
+    m.jx = (D[1] - D[3]) + (d57 - d68);
+    m.jy = (D[2] - D[4]) + (d57 + d68);
+    m.pxy = s57 - s68;
+    m.del = a13 - a24;
+    m.s32 = (a1324 >> 1) + 2 * sd - D[0];
+    return m;
+}
+
+// The common exponent of a node's populations; false when it leaves the range.
+BTRT_HD bool fx_common_exp(const double (&d)[9], unsigned int &em) {
+    em = kFxExpMin;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const unsigned int e = fx_exp(d[i]);
+        em = em > e ? em : e;
+    }
+    return em <= kFxExpMax;
+}
+
+// The outputs of a node, (1 - k0) D_i + r_i, as FP64; the first NADD by the FP64
+// adder (fx_to_add), the others by integer instructions.
+template <bool K0ONE, int NADD>
+BTRT_HD void fx_store(const fx (&D)[9], const fx (&r)[9], const FxConst &om2, unsigned int em, double (&d)[9]) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const fx v = K0ONE ? r[i] : r[i] + 2 * fx_mul(fx_arg(D[i]), om2);
+        d[i] = i < NADD ? fx_to_add(v, em) : fx_to(v, em);
+    }
+}
+
+// Populations that the FP64 adder converts in the constant-coefficient collision:
+// the 8192^2 manufactured solution (20 steps) measured 52.7 / 49.0 / 49.4 ms with 0 / 3 / 5
+// (four rows per thread) and 38.8 / 38.2 / 42.0 with 4 / 5 / 6 at six blocks per SM,
+// 37.5 / 38.1 with 4 / 5 at five.
+#ifndef BTRT_FX_NADD
+#define BTRT_FX_NADD 4
+#endif
+
+// The constant-coefficient collision of one node: d in, post-collision populations
+// out; src is the node's source term (0 when there is none).  Returns false, with
+// d untouched, when the node's values leave the range (the caller takes the FP64
+// form): the exponents of the populations, or phi^{n-1} or the source more than four
+// times or twice the largest population.
+template <bool K0ONE, bool SOURCE>
+BTRT_HD bool fx_collide_linear(const FxFold &q, double (&d)[9], double phi_prev, double src, double &phi_out) {
+    unsigned int em;
+    if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;
+    if (SOURCE && fx_exp(src) > em + (1u << 20)) return false;
+    fx D[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) D[i] = fx_from(d[i], em);
+    const FxMoments m = fx_moments(D);
+    const FxArg jx = fx_arg(m.jx), jy = fx_arg(m.jy), ph = fx_arg(m.phi), pp = fx_arg(fx_from(phi_prev, em));
+    FxSum sx = fx_sum(), sy = fx_sum();
+    fx_add(sx, jx, q.Qxx);
+    fx_add(sx, jy, q.Qxy);
+    fx_add(sx, ph, q.Px);
+    fx_add(sx, pp, q.gx);
+    fx_add(sy, jx, q.Qxy);
+    fx_add(sy, jy, q.Qyy);
+    fx_add(sy, ph, q.Py);
+    fx_add(sy, pp, q.gy);
+    const fx ks = fx_mul(fx_arg(m.s32), q.d18), t1 = fx_mul(fx_arg(m.del), q.d4), t5 = fx_mul(fx_arg(m.pxy), q.d4);
+    fx a = m.phi;
+    if (!K0ONE) a -= 2 * fx_mul(ph, q.om2);
+    if (SOURCE) a += fx_from(src, em);
+    fx r[9];
+    fx_expand(a, 0, fx_value(sx), fx_value(sy), ks, t1, t5, r);
+    fx_store<K0ONE, BTRT_FX_NADD>(D, r, q.om2, em, d);
+    phi_out = fx_to(m.phi, em);
+    return true;
+}
+
+}  // namespace btrt

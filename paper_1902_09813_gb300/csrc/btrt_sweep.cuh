@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "btrt_dw.cuh"
+#include "btrt_fx.cuh"
 
 namespace btrt {
 
@@ -95,9 +96,15 @@ struct FoldConsts {
     Real a2x3;             // 3 a2                   (phi-dependent coefficients)
 };
 
+// Constants of the integer collision: FP64 lattices only (an empty base elsewhere).
+template <typename Real> struct FxPart {};
+template <> struct FxPart<double> {
+    FxFold fx;
+};
+
 // Everything one launch of the sweep needs, passed by value.
 template <typename Real>
-struct SweepParams {
+struct SweepParams : FxPart<Real> {
     const void *fin;       // post-collision populations at step n-1: 9 planes, `plane` apart
     void *fout;            // post-collision populations at step n
     const Real *phi_in;    // phi^{n-1} (the phi of the nodes that wrote fin)
@@ -266,15 +273,15 @@ static __device__ __noinline__ K1f k1_fp64(double phi, double a2, double bxx, do
     return K1f{(float)(dyy * id), (float)(-dxy * id), (float)(dxx * id)};
 }
 
-// FP64 operations (add, multiply or FMA: one each) per node of the FP64 sweep in
-// its k0 = 1 constant-coefficient form with the trig source
-// (sweep_kernel<double, double, kShiftNone, kLinearK0One, kSrcTrig>), counted
-// from collide_fold and source_at below: the moments 18 adds (a13, a24, s57,
-// s68, sd, a1324, phid, b13, b24, d57, d68, jx: 2, jy: 2, pxy, del), V 2 adds
-// (Vp, Vm); qx, qy 2 FMAs + 2 multiplies, Vx, Vy 4 FMAs, sig 2 FMAs, r0 1 FMA +
-// 1 multiply, ks 1 multiply, T1, T5 2 FMAs, A1, A2, P, M 4 FMAs, r1..r8 8 FMAs,
-// the trig source 1 FMA + 1 multiply and a = ... + src 1 FMA: 20 adds, 25 FMAs,
-// 5 multiplies.  ncu counts 50.6 per node (DADD 20.5, DFMA 25.0, DMUL 5.0).
+// FP64 operations (add, multiply or FMA: one each) per node of collide_fold in its
+// k0 = 1 constant-coefficient form with the trig source, the scheme's count that the
+// benchmark reports: the moments 18 adds (a13, a24, s57, s68, sd, a1324, phid, b13,
+// b24, d57, d68, jx: 2, jy: 2, pxy, del), V 2 adds (Vp, Vm); qx, qy 2 FMAs + 2
+// multiplies, Vx, Vy 4 FMAs, sig 2 FMAs, r0 1 FMA + 1 multiply, ks 1 multiply, T1,
+// T5 2 FMAs, A1, A2, P, M 4 FMAs, r1..r8 8 FMAs, the trig source 1 FMA + 1 multiply
+// and a = ... + src 1 FMA: 20 adds, 25 FMAs, 5 multiplies.  The FP64 sweep keeps 11
+// of them on the FP64 pipe (the source, and two additions for each of the four
+// populations converted by fx_to_add); the rest is integer arithmetic (collide_f64).
 constexpr int kFp64AddsPerNodeLinearTrig = 20;
 constexpr int kFp64FmasPerNodeLinearTrig = 25;
 constexpr int kFp64MulsPerNodeLinearTrig = 5;
@@ -458,6 +465,217 @@ __device__ __forceinline__ Real collide_fold(const SweepParams<Real> &p, Real (&
     return phi;
 }
 
+// ---------------------------------------------------------------- the FP64 collision on the integer pipes
+// The FP64 form of collide_fold for one node, out of line: the nodes whose values
+// the integer form does not take, and the initialising collision.
+template <int MODE, int SRC>
+static __device__ __noinline__ double collide_f64_slow(const SweepParams<double> &p, double *t, double phi_prev,
+                                                       double srcv, int node) {
+    double d[9], phid;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) d[i] = t[i];
+    const double phi = collide_fold<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, node, phid);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) t[i] = d[i];
+    return phi;
+}
+
+// 1/v by Householder's third-order iteration on the hardware's approximate
+// reciprocal (relative error e below 2^-18): x (1 + e + e^2), error e^3 plus the
+// rounding of the last step.
+__device__ __forceinline__ double recip_f64(double v) {
+    double x;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(v));
+    const double e = fma(-v, x, 1.0);
+    return fma(x, fma(e, e, e), x);
+}
+
+// The per-node coefficient collision (kGeneral), or a reaction source: the moments
+// and the populations are integers as in fx_collide_linear, the nonlinear
+// coefficients and V are FP64 (44 operations instead of 97 with the two divisions
+// sharing one reciprocal).  Returns false, with d untouched, when a value leaves
+// the integer form's range.
+template <int MODE, int SRC>
+__device__ __forceinline__ bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], double phi_prev,
+                                                   double srcv, int node, double &phi_out) {
+    const FoldConsts<double> &L = p.lin;
+    unsigned int em;
+    if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;
+    fx D[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) D[i] = fx_from(d[i], em);
+    FxMoments m = fx_moments(D);
+    const double phi = fx_to(m.phi, em);
+    fx X, Y, z = 0;
+    FxConst d4, d18;
+    if constexpr (MODE == kGeneral) {
+        const double jx = fx_to(m.jx, em), jy = fx_to(m.jy, em);
+        const double dphi = phi - phi_prev;
+        const double p2 = phi * phi;
+        double Bx, By, dBx, dBy;
+        if (p.bq2) {
+            Bx = fma(p.ux, phi, p.bgx * p2);
+            By = fma(p.uy, phi, p.bgy * p2);
+            const double sp = phi + phi_prev;
+            dBx = fma(p.bgx, sp, p.ux) * dphi;
+            dBy = fma(p.bgy, sp, p.uy) * dphi;
+        } else {
+            const double gq = pow_half(phi, p.bq, p.bq_n, p.bq_h);
+            const double dg = gq - pow_half(phi_prev, p.bq, p.bq_n, p.bq_h);
+            Bx = fma(p.ux, phi, p.bgx * gq);
+            By = fma(p.uy, phi, p.bgy * gq);
+            dBx = fma(p.ux, dphi, p.bgx * dg);
+            dBy = fma(p.uy, dphi, p.bgy * dg);
+        }
+        if (p.c3 != 0.0) {
+            // C(phi) - phi: in sigma, and k0 (C - phi) / 18 in the isotropic terms
+            const double Cm = p.c3 * p2 * phi;
+            if (fx_exp(Cm) > em + (1u << 20)) return false;
+            m.s32 -= fx_from(Cm, em);
+            z = fx_from(p.k0 * cst<double>(1, 18) * Cm, em);
+        }
+        const double s3 = fma(L.a2x3, p2, 3.0);
+        double a0xx = p.A0xx, a0xy = p.A0xy, a0yy = p.A0yy;
+        if (p.Af) {
+            a0xx = p.Af[BTRT_IX(p.flags, node, p.plane)];
+            a0xy = p.Af[BTRT_IX(p.flags, p.plane + node, 3 * p.plane)];
+            a0yy = p.Af[BTRT_IX(p.flags, 2 * p.plane + node, 3 * p.plane)];
+        }
+        const double mxx = fma(s3, a0xx, 0.5), mxy = s3 * a0xy, myy = fma(s3, a0yy, 0.5);
+        const double tr = mxx + myy;
+        const double det = fma(mxx, myy, -(mxy * mxy));
+        double id, k2;
+        if (p.k2_hbb) {
+            const double q2 = fma(2.0, tr, -1.0);
+            const double rc = recip_f64(det * q2);
+            id = rc * q2;
+            k2 = (fma(cst<double>(8, 3), tr, -cst<double>(8, 3)) * det) * rc;
+        } else {
+            id = recip_f64(det);
+            k2 = p.k2c;
+        }
+        const double dk = k2 - p.k0;
+        const double ex = fma(-0.5, dBx, Bx - jx), ey = fma(-0.5, dBy, By - jy);
+        const double Kxx = myy * id, Kxy = -mxy * id, Kyy = mxx * id;
+        const double Vx = fma(Kxx, ex, fma(Kxy, ey, fma(p.k0, jx, dBx)));
+        const double Vy = fma(Kxy, ex, fma(Kyy, ey, fma(p.k0, jy, dBy)));
+        // also false for infinities and NaN
+        if (fx_exp(dk) > (1023u << 20) || fx_exp(Vx) > em + (2u << 20) || fx_exp(Vy) > em + (2u << 20)) return false;
+        const FxConst sixth = {0x2aaaaaab, (int)0xaaaaaaab};   // 2^64 / 6
+        X = fx_mul(fx_arg(fx_from(Vx, em)), sixth);
+        Y = fx_mul(fx_arg(fx_from(Vy, em)), sixth);
+        const FxArg c = fx_arg(fx_from(dk, 1019u << 20));      // dk / 4 in units of 2^-64
+        d4.hi = c.h;
+        d4.lo = c.l;
+        d18 = d4;
+        m.s32 = 2 * fx_ninth(m.s32);                           // (k2 - k0)/18 = (2/9) (k2 - k0)/4
+    } else {
+        const FxArg jx = fx_arg(m.jx), jy = fx_arg(m.jy), ph = fx_arg(m.phi), pp = fx_arg(fx_from(phi_prev, em));
+        FxSum sx = fx_sum(), sy = fx_sum();
+        fx_add(sx, jx, p.fx.Qxx);
+        fx_add(sx, jy, p.fx.Qxy);
+        fx_add(sx, ph, p.fx.Px);
+        fx_add(sx, pp, p.fx.gx);
+        fx_add(sy, jx, p.fx.Qxy);
+        fx_add(sy, jy, p.fx.Qyy);
+        fx_add(sy, ph, p.fx.Py);
+        fx_add(sy, pp, p.fx.gy);
+        X = fx_value(sx);
+        Y = fx_value(sy);
+        d4 = p.fx.d4;
+        d18 = p.fx.d18;
+    }
+    double src = 0.0;
+    if constexpr (SRC == kSrcReaction || SRC == kSrcRuntime) {
+        if (SRC == kSrcReaction || p.src_kind == kSrcReaction)
+            srcv = fma(1.5, reaction(p, phi), -0.5 * reaction(p, phi_prev));
+    }
+    if constexpr (SRC != kSrcNone) src = p.src_val * srcv;
+    if (SRC != kSrcNone && fx_exp(src) > em + (1u << 20)) return false;
+    const fx ks = fx_mul(fx_arg(m.s32), d18), t1 = fx_mul(fx_arg(m.del), d4), t5 = fx_mul(fx_arg(m.pxy), d4);
+    fx a = m.phi, r[9];
+    const bool k0_one = MODE == kLinearK0One || p.k0_one;
+    if (!k0_one) a -= 2 * fx_mul(fx_arg(m.phi), p.fx.om2);
+    if (SRC != kSrcNone) a += fx_from(src, em);
+    fx_expand(a, z, X, Y, ks, t1, t5, r);
+    // the FP64 pipe bounds the per-node coefficients; the constant ones are converted as in
+    // fx_collide_linear (ties round differently in the two conversions)
+    constexpr int NADD = MODE == kGeneral ? 0 : BTRT_FX_NADD;
+    if (k0_one) fx_store<true, NADD>(D, r, p.fx.om2, em, d);
+    else fx_store<false, NADD>(D, r, p.fx.om2, em, d);
+    phi_out = phi;
+    return true;
+}
+
+// The initialising collision of one node: the equilibrium of phi has no
+// non-equilibrium moments, so the collision leaves it and adds the source,
+// f_i = f_i^eq + w_i S: a = phi + S, V = B and C in fx_expand.  FP64 out of line as
+// above where a value leaves the range.
+template <int MODE, int SRC>
+static __device__ __noinline__ void init_f64_slow(const SweepParams<double> &p, double *t, double phi, double src);
+template <int MODE, int SRC>
+__device__ __forceinline__ void init_f64(const SweepParams<double> &p, double (&d)[9], double phi, double src) {
+    double Bx = p.ux * phi, By = p.uy * phi, Cm = 0.0;
+    if constexpr (MODE == kGeneral) {
+        const double g = flux_pow(p, phi);
+        Bx = fma(p.bgx, g, Bx);
+        By = fma(p.bgy, g, By);
+        Cm = p.c3 * phi * phi * phi;
+    }
+    unsigned int em = fx_exp(phi);
+    em = em > kFxExpMin ? em : kFxExpMin;
+    const unsigned int far = em + (1u << 20);
+    if (em > kFxExpMax || fx_exp(Bx) > far || fx_exp(By) > far || fx_exp(src) > far || fx_exp(Cm) > far) {
+        double t[9];
+        init_f64_slow<MODE, SRC>(p, t, phi, src);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) d[i] = t[i];
+        return;
+    }
+    const FxConst sixth = {0x2aaaaaab, (int)0xaaaaaaab};   // 2^64 / 6
+    fx a = fx_from(phi, em), z = 0, r[9];
+    if (SRC != kSrcNone) a += fx_from(src, em);
+    if (MODE == kGeneral) z = fx_from(cst<double>(1, 18) * Cm, em);
+    fx_expand(a, z, fx_mul(fx_arg(fx_from(Bx, em)), sixth), fx_mul(fx_arg(fx_from(By, em)), sixth), 0, 0, 0, r);
+    fx_store<true, BTRT_FX_NADD>(r, r, p.fx.om2, em, d);
+}
+
+// The FP64 collision of one node: the integer form, or the FP64 one where the
+// integer form does not serve (a value out of its range, constants that do not
+// fit).  FP64 alone: 0.985 of the FP64 pipe at 10.4 GLUPS on the 8192^2
+// manufactured solution, 5.55 on the nonlinear workload; with the integer form
+// 37 GLUPS (0.89 of HBM) and 10.8.
+template <int MODE, int SRC>
+__device__ __forceinline__ double collide_f64(const SweepParams<double> &p, double (&d)[9], double phi_prev,
+                                              double srcv, int node) {
+    constexpr bool LATE = SRC == kSrcReaction || SRC == kSrcRuntime;   // the source may depend on phi
+    if (p.first) {
+        double src = SRC != kSrcNone ? p.src_val * srcv : 0.0;
+        if (LATE && (SRC == kSrcReaction || p.src_kind == kSrcReaction)) src = p.src_val * reaction(p, phi_prev);
+        init_f64<MODE, SRC>(p, d, phi_prev, src);
+        return phi_prev;
+    }
+    double phi;
+    bool done = false;
+    if (p.fx.ok & (MODE == kGeneral ? kFxOkGeneral : kFxOkLinear)) {
+        if constexpr (MODE == kGeneral || LATE)
+            done = fx_collide_general<MODE, SRC>(p, d, phi_prev, srcv, node, phi);
+        else if (MODE == kLinearK0One || p.k0_one)
+            done = fx_collide_linear<true, SRC != kSrcNone>(p.fx, d, phi_prev, SRC != kSrcNone ? p.src_val * srcv : 0.0, phi);
+        else
+            done = fx_collide_linear<false, SRC != kSrcNone>(p.fx, d, phi_prev, SRC != kSrcNone ? p.src_val * srcv : 0.0, phi);
+    }
+    if (!done) {
+        double t[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) t[i] = d[i];
+        phi = collide_f64_slow<MODE, SRC>(p, t, phi_prev, srcv, node);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) d[i] = t[i];
+    }
+    return phi;
+}
+
 // Equilibrium populations (Eq. 7) in lattice units, D = C(phi) I, shifted by
 // w_i rs as the collision expects (rs = phi for the local shift).
 template <typename Real, int SH>
@@ -485,6 +703,14 @@ __device__ __forceinline__ void equilibrium(const SweepParams<Real> &p, Real phi
 #pragma unroll
         for (int i = 0; i < 9; ++i) f[i] = fma(-wgt<Real>(i), phi, f[i]);
     }
+}
+
+template <int MODE, int SRC>
+static __device__ __noinline__ void init_f64_slow(const SweepParams<double> &p, double *t, double phi, double src) {
+    double d[9];
+    equilibrium<double, kShiftNone>(p, phi, d);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) t[i] = fma(wgt<double>(i), src, d[i]);
 }
 
 // Non-finite test without touching the FP64 pipe: exponent field all ones.
@@ -598,8 +824,9 @@ template <typename S, int SH> struct ShiftOf { static constexpr int value = SH; 
 template <int SH> struct ShiftOf<double, SH> { static constexpr int value = kShiftNone; };
 template <int SH> struct ShiftOf<dw, SH> { static constexpr int value = kShiftNone; };
 
-// Nodes per thread of the single-lattice sweep: the FP64 sweep is ALU-bound and
-// amortises per-thread set-up over a column of 4 nodes; the HBM-bound FP32-storage
+// Nodes per thread of the single-lattice sweep: one for FP64 (a column of 4 measured
+// 49.4 ms against 47.8 on the 8192^2 manufactured solution, and 3.65 against 3.14 on
+// the 1001 x 777 nonlinear workload, whose last wave it leaves half empty); the HBM-bound FP32-storage
 // sweep takes two nodes with both pulls issued before the collisions (loads in
 // flight together, set-up shared); the FP16/BF16-storage sweeps, limited by
 // registers and issue, keep one node per thread.  The BTRT_ROWS_* macros
@@ -625,10 +852,10 @@ template <> struct RowsPerThread<float, float> {
     static constexpr bool unroll = BTRT_UNROLL_S32 != 0;
 };
 #ifndef BTRT_ROWS_F64
-#define BTRT_ROWS_F64 4
+#define BTRT_ROWS_F64 1
 #endif
 #ifndef BTRT_MINBLOCKS_F64
-#define BTRT_MINBLOCKS_F64 0
+#define BTRT_MINBLOCKS_F64 5
 #endif
 #ifndef BTRT_UNROLL_F64
 #define BTRT_UNROLL_F64 0
@@ -648,11 +875,14 @@ template <> struct RowsPerThread<double, double> {
 #endif
 // Minimum resident blocks per SM requested from the compiler (register budget);
 // 0 leaves the choice to the compiler.
-// FP64 per-node coefficient sweeps: the compiler's 96 registers (two blocks);
-// four blocks (64 registers) measured 5.14 GLUPS against 5.57 on the nonlinear
-// workload.
+// FP64 sweeps run on the integer pipes and need warps to cover load latency: five
+// blocks (48 registers) for k0 = 1 with constant coefficients measured 37.5 ms on
+// the 8192^2 manufactured solution (20 steps and the set-up), six 38.8; other k0 and
+// a reaction source would spill there, four and three blocks do not.  Per-node
+// coefficients: three blocks (80 registers), 2.95 ms on the 1001 x 777 nonlinear
+// workload against 3.14 with two.
 #ifndef BTRT_MINBLOCKS_F64_GEN
-#define BTRT_MINBLOCKS_F64_GEN 0
+#define BTRT_MINBLOCKS_F64_GEN 3
 #endif
 // Double-word constant-coefficient sweeps: five blocks (48 registers, 12 spilled
 // bytes) measured 36.9 GLUPS against 33.5 with the compiler's 64 registers; the
@@ -660,14 +890,16 @@ template <> struct RowsPerThread<double, double> {
 #ifndef BTRT_MINBLOCKS_DW
 #define BTRT_MINBLOCKS_DW 5
 #endif
-template <typename Real, typename S, int MODE> struct MinBlocks { static constexpr int value = 0; };
-template <int MODE> struct MinBlocks<double, double, MODE> {
-    static constexpr int value = MODE == kGeneral ? BTRT_MINBLOCKS_F64_GEN : BTRT_MINBLOCKS_F64;
+template <typename Real, typename S, int MODE, int SRC> struct MinBlocks { static constexpr int value = 0; };
+template <int MODE, int SRC> struct MinBlocks<double, double, MODE, SRC> {
+    static constexpr int value = MODE == kGeneral || SRC == kSrcReaction ? BTRT_MINBLOCKS_F64_GEN
+                                 : MODE == kLinearK0One                  ? BTRT_MINBLOCKS_F64
+                                                                         : 4;
 };
-template <int MODE> struct MinBlocks<float, float, MODE> { static constexpr int value = BTRT_MINBLOCKS_F32; };
-template <int MODE> struct MinBlocks<float, __half, MODE> { static constexpr int value = BTRT_MINBLOCKS_S16; };
-template <int MODE> struct MinBlocks<float, __nv_bfloat16, MODE> { static constexpr int value = BTRT_MINBLOCKS_S16; };
-template <int MODE> struct MinBlocks<dw, dw, MODE> {
+template <int MODE, int SRC> struct MinBlocks<float, float, MODE, SRC> { static constexpr int value = BTRT_MINBLOCKS_F32; };
+template <int MODE, int SRC> struct MinBlocks<float, __half, MODE, SRC> { static constexpr int value = BTRT_MINBLOCKS_S16; };
+template <int MODE, int SRC> struct MinBlocks<float, __nv_bfloat16, MODE, SRC> { static constexpr int value = BTRT_MINBLOCKS_S16; };
+template <int MODE, int SRC> struct MinBlocks<dw, dw, MODE, SRC> {
     static constexpr int value = MODE == kGeneral ? 0 : BTRT_MINBLOCKS_DW;
 };
 template <> struct RowsPerThread<dw, dw> { static constexpr int value = 1; static constexpr bool unroll = false; };
@@ -678,6 +910,23 @@ template <bool L2ONLY, typename T>
 __device__ __forceinline__ T ldg(const T *ptr) {
     if constexpr (L2ONLY) return __ldcg(ptr);
     else return *ptr;
+}
+
+// Element `at` of population plane i.  FP64: the plane's base is uniform over the
+// launch and the element's byte offset fits 32 bits (9 planes hold fewer than 2^31
+// values), so one 32-bit offset serves every plane.
+template <typename Real, typename S>
+__device__ __forceinline__ const S *plane_at(const SweepParams<Real> &p, const S *f, int i, int at) {
+#ifndef BTRT_DEBUG_BOUNDS
+    if constexpr (std::is_same<Real, double>::value)
+        return reinterpret_cast<const S *>(reinterpret_cast<const char *>(f + (size_t)i * p.plane) +
+                                           (unsigned int)at * (unsigned int)sizeof(S));
+#endif
+    return f + BTRT_IX(p.flags, i * p.plane + at, 9 * p.plane);
+}
+template <typename Real, typename S>
+__device__ __forceinline__ S *plane_at(const SweepParams<Real> &p, S *f, int i, int at) {
+    return const_cast<S *>(plane_at<Real, S>(p, const_cast<const S *>(f), i, at));
 }
 
 // Pull of a node on the domain boundary: periodic wrap or, for a link that
@@ -772,13 +1021,13 @@ __device__ __forceinline__ void pull_node(const SweepParams<Real> &p, int x, int
         phi_lo = ldg<L2ONLY>(p.phi_in_lo + BTRT_IX(p.flags, node, p.plane));
         *phi_lo_out = phi_lo;
     }
-    if (p.first) {
-        equilibrium<Real, CollShift<SH>::value>(p, phi_prev, f);
+    if (p.first) {   // FP64: formed in the collision (init_f64)
+        if constexpr (!std::is_same<Real, double>::value) equilibrium<Real, CollShift<SH>::value>(p, phi_prev, f);
     } else if (x_inner && y > 0 && y < p.ny - 1) {
 #pragma unroll
         for (int i = 0; i < 9; ++i)
             f[i] = dev_load<Real, S, SH>(
-                ldg<L2ONLY>(fin + BTRT_IX(p.flags, i * p.plane + node - ey_of(i) * p.pitch - ex_of(i), 9 * p.plane)));
+                ldg<L2ONLY>(plane_at<Real, S>(p, fin, i, node - ey_of(i) * p.pitch - ex_of(i))));
         if constexpr (PS == kShiftLocal || PS == kShiftMomentSR) {
 #pragma unroll
             for (int i = 1; i < 9; ++i)
@@ -830,8 +1079,13 @@ __device__ __forceinline__ double finish_node(const SweepParams<Real> &p, int x,
     const int node = y * p.pitch + x;
     const Real src = source_at<Real, SRC>(p, xs, xc, y, node);
     const Real rs = SC == kShiftLocal ? phi_prev : p.phi_ref;
-    Real phid;
-    const Real phi = collide_fold<Real, MODE, SRC, SC>(p, f, rs, phi_prev, src, p.first != 0, node, phid, Lc);
+    Real phid, phi;
+    if constexpr (std::is_same<Real, double>::value) {
+        phi = collide_f64<MODE, SRC>(p, f, phi_prev, src, node);
+        phid = phi;
+    } else {
+        phi = collide_fold<Real, MODE, SRC, SC>(p, f, rs, phi_prev, src, p.first != 0, node, phid, Lc);
+    }
     if constexpr (PullShift<SH>::value == kShiftMomentSR) {
         // the writer's first moment sum_i e_i d_i^+ (the w_i rs terms cancel), stored
         // rounded; the deviations are taken from w_i (phi + 3 e_i . j) with the stored j
@@ -856,7 +1110,7 @@ __device__ __forceinline__ double finish_node(const SweepParams<Real> &p, int x,
             fout[BTRT_IX(p.flags, i * p.plane + node, 9 * p.plane)] = pack_sr<S>(fma(-wgt<Real>(i), phid, f[i]), sr_bits(h, i));
     } else {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) fout[BTRT_IX(p.flags, i * p.plane + node, 9 * p.plane)] = store_value<Real, S, SC>(i, f[i], phid);
+        for (int i = 0; i < 9; ++i) *plane_at<Real, S>(p, fout, i, node) = store_value<Real, S, SC>(i, f[i], phid);
     }
     if constexpr (PullShift<SH>::value == kShiftLocalDW) {
         // phi^n = (phi_prev + phi_lo) + phid as a double-word pair: TwoSum of the high
@@ -939,7 +1193,7 @@ __device__ __forceinline__ double sweep_rows(const SweepParams<Real> &p, int x, 
 // One sweep of one lattice: 32 x 8 threads per block, each thread sweeps
 // RowsPerThread nodes of its column, rows blockDim.y apart.
 template <typename Real, typename S, int SH, int MODE, int SRC>
-__global__ void __launch_bounds__(256, MinBlocks<Real, S, MODE>::value) sweep_kernel(const __grid_constant__ SweepParams<Real> p) {
+__global__ void __launch_bounds__(256, MinBlocks<Real, S, MODE, SRC>::value) sweep_kernel(const __grid_constant__ SweepParams<Real> p) {
     constexpr int R = RowsPerThread<Real, S>::value;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int ybase = blockIdx.y * blockDim.y * R + threadIdx.y;
