@@ -75,13 +75,14 @@ BTRT_HD double fx_double(unsigned long long b) {
 // Exponent field of v, in place in the high word.
 BTRT_HD unsigned int fx_exp(double v) { return (unsigned int)(fx_bits(v) >> 32) & kFxExpMask; }
 
-// v in units of 2^(E - 58) (E = em >> 20, biased as in FP64), truncated toward
+// v in units of 2^(E - TOP) (E = em >> 20, biased as in FP64), truncated toward
 // zero: the mantissa with its hidden bit at the top of the word, shifted down by
-// E + 5 - e.  Shifts of 64 and more give 0 (also for zeros and subnormals, whose
-// hidden bit is not there: E >= 64 shifts them out).  e <= E + 4.
-BTRT_HD fx fx_from(double v, unsigned int em) {
+// E + 63 - TOP - e.  D2Q9: TOP = 58, nine populations then sum below 2^63; D3Q19: 57.
+// Shifts of 64 and more give 0 (also for zeros and subnormals, whose
+// hidden bit is not there: E >= 64 shifts them out).  e <= E + 62 - TOP.
+template <int TOP = 58> BTRT_HD fx fx_from(double v, unsigned int em) {
     const unsigned long long b = fx_bits(v);
-    const unsigned int sh = (em + (5u << 20) - ((unsigned int)(b >> 32) & kFxExpMask)) >> 20;
+    const unsigned int sh = (em + ((63u - TOP) << 20) - ((unsigned int)(b >> 32) & kFxExpMask)) >> 20;
     unsigned long long m = (b << 11) | 0x8000000000000000ull;
 #ifdef __CUDA_ARCH__
     asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(sh));   // PTX clamps the amount at 64
@@ -92,11 +93,11 @@ BTRT_HD fx fx_from(double v, unsigned int em) {
     return ((fx)m ^ s) - s;
 }
 
-// The FP64 value nearest to v 2^(E - 58) (ties away from zero).
-BTRT_HD double fx_to(fx v, unsigned int em) {
+// The FP64 value nearest to v 2^(E - TOP) (ties away from zero).
+template <int TOP = 58> BTRT_HD double fx_to(fx v, unsigned int em) {
     const fx s = v >> 63;
     const unsigned long long a = (unsigned long long)((v ^ s) - s);
-    unsigned int hi = (unsigned int)(a >> 32), lo = (unsigned int)a, up = em + (4u << 20);
+    unsigned int hi = (unsigned int)(a >> 32), lo = (unsigned int)a, up = em + ((62u - TOP) << 20);
     if (hi == 0) {
         hi = lo;
         lo = 0;
@@ -121,14 +122,14 @@ BTRT_HD double fx_to(fx v, unsigned int em) {
 // mantissas of 2^84 and 2^52, the constants leave again, and only the second
 // addition rounds.  The FP64 adder is otherwise idle here, but ten conversions
 // would make it the bound.
-BTRT_HD double fx_to_add(fx v, unsigned int em) {
+template <int TOP = 58> BTRT_HD double fx_to_add(fx v, unsigned int em) {
     const unsigned long long u = (unsigned long long)v;
     const double b = fx_double(0x4530000000000000ull | ((u >> 32) ^ 0x80000000ull));
     const double a = fx_double(0x4330000000000000ull | (u & 0xffffffffull));
     const double r = (b - 19342822341709703277445120.0) + a;   // 2^84 + 2^63 + 2^52
     const unsigned long long rb = fx_bits(r);
     const unsigned int rh = (unsigned int)(rb >> 32);
-    return fx_double((unsigned long long)(rh ? rh + em - (1081u << 20) : 0u) << 32 | (rb & 0xffffffffull));
+    return fx_double((unsigned long long)(rh ? rh + em - ((1023u + TOP) << 20) : 0u) << 32 | (rb & 0xffffffffull));
 }
 
 // x as h 2^32 + l with l signed, for the products below.
@@ -236,10 +237,10 @@ BTRT_HD FxMoments fx_moments(const fx (&D)[9]) {
 }
 
 // The common exponent of a node's populations; false when it leaves the range.
-BTRT_HD bool fx_common_exp(const double (&d)[9], unsigned int &em) {
+template <int N> BTRT_HD bool fx_common_exp(const double (&d)[N], unsigned int &em) {
     em = kFxExpMin;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
+    for (int i = 0; i < N; ++i) {
         const unsigned int e = fx_exp(d[i]);
         em = em > e ? em : e;
     }
@@ -248,12 +249,12 @@ BTRT_HD bool fx_common_exp(const double (&d)[9], unsigned int &em) {
 
 // The outputs of a node, (1 - k0) D_i + r_i, as FP64; the first NADD by the FP64
 // adder (fx_to_add), the others by integer instructions.
-template <bool K0ONE, int NADD>
-BTRT_HD void fx_store(const fx (&D)[9], const fx (&r)[9], const FxConst &om2, unsigned int em, double (&d)[9]) {
+template <bool K0ONE, int NADD, int TOP = 58, int N>
+BTRT_HD void fx_store(const fx (&D)[N], const fx (&r)[N], const FxConst &om2, unsigned int em, double (&d)[N]) {
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
+    for (int i = 0; i < N; ++i) {
         const fx v = K0ONE ? r[i] : r[i] + 2 * fx_mul(fx_arg(D[i]), om2);
-        d[i] = i < NADD ? fx_to_add(v, em) : fx_to(v, em);
+        d[i] = i < NADD ? fx_to_add<TOP>(v, em) : fx_to<TOP>(v, em);
     }
 }
 
@@ -297,6 +298,138 @@ BTRT_HD bool fx_collide_linear(const FxFold &q, double (&d)[9], double phi_prev,
     fx_expand(a, 0, fx_value(sx), fx_value(sy), ks, t1, t5, r);
     fx_store<K0ONE, BTRT_FX_NADD>(D, r, q.om2, em, d);
     phi_out = fx_to(m.phi, em);
+    return true;
+}
+
+// ---------------------------------------------------------------- D3Q19
+// Velocity order as in btrt_sweep3.cuh: rest; +-x, +-y, +-z; xy, xz and yz diagonals
+// with signs (+,+) (-,+) (+,-) (-,-).  Units of 2^(E - 57): nineteen populations
+// below 2^58 sum below 2^63.
+constexpr int kFxTop3 = 57;
+
+// V/6 takes -(K1 - k0 I)/6 on the first moments, (K1 u^ + g)/6 on phi, -g/6 on
+// phi^{n-1}; (k2 - k0)/12 acts on 3 h_a, (k2 - k0)/24 on 3 t3, (k2 - k0)/4 on Pi_ab
+// (collide3 for the scheme and the names).
+struct FxFold3 {
+    FxConst Q[6];    // xx, xy, xz, yy, yz, zz
+    FxConst P[3], g[3], d12, d24, d4, om2;
+    int ok;          // kFxOk* bits
+    int pad;
+};
+
+// As fx_flux_fits: populations below 2^58 units, phi^{n-1} below 2^61.
+inline bool fx_flux_fits3(const FxConst &qx, const FxConst &qy, const FxConst &qz, const FxConst &cp, const FxConst &cg) {
+    auto mag = [](double v) { return v < 0 ? -v : v; };
+    double t = 17179869184.0 + 536870912.0 * mag(cg.lo);
+    for (int x = -1; x <= 1; ++x)
+        for (int y = -1; y <= 1; ++y)
+            for (int z = -1; z <= 1; ++z)
+                if (x * x + y * y + z * z <= 2)
+                    t += 67108864.0 * mag((double)x * qx.lo + (double)y * qy.lo + (double)z * qz.lo + cp.lo);
+    t += 2147483648.0 * (mag(qx.hi) + mag(qy.hi) + mag(qz.hi) + mag(cp.hi) + mag(cg.hi) + 5.0);
+    return t < 9223372036854775808.0;
+}
+
+struct FxMoments3 {
+    fx phi, jx, jy, jz, pxy, pxz, pyz;
+    fx hx, hy, t3;   // 3 h_x, 3 h_y (h_z = -h_x - h_y) and 3 t3
+};
+BTRT_HD FxMoments3 fx_moments3(const fx (&D)[19]) {
+    FxMoments3 m;
+    const fx ax = D[1] + D[2], ay = D[3] + D[4], az = D[5] + D[6];
+    const fx xyp = D[7] + D[8], xym = D[9] + D[10], xyd = D[7] - D[8], xye = D[9] - D[10];
+    const fx xzp = D[11] + D[12], xzm = D[13] + D[14], xzd = D[11] - D[12], xze = D[13] - D[14];
+    const fx yzp = D[15] + D[16], yzm = D[17] + D[18], yzd = D[15] - D[16], yze = D[17] - D[18];
+    const fx sxy = xyp + xym, sxz = xzp + xzm, syz = yzp + yzm;
+    m.jx = (D[1] - D[2]) + (xyd + xye) + (xzd + xze);
+    m.jy = (D[3] - D[4]) + (xyp - xym) + (yzd + yze);
+    m.jz = (D[5] - D[6]) + (xzp - xzm) + (yzp - yzm);
+    m.pxy = xyd - xye;
+    m.pxz = xzd - xze;
+    m.pyz = yzd - yze;
+    const fx Pxx = ax + sxy + sxz, Pyy = ay + sxy + syz, Pzz = az + sxz + syz;
+    const fx S = Pxx + Pyy + Pzz, sd = sxy + sxz + syz;
+    m.phi = D[0] + (S - sd);            // the diagonals count twice in S
+    m.hx = 2 * Pxx - Pyy - Pzz;
+    m.hy = 2 * Pyy - Pxx - Pzz;
+    m.t3 = sd - D[0];                   // S - phi
+    return m;
+}
+
+// Populations from a = k0 phi + source, z (the term of C(phi) != phi on the diagonals),
+// X = V/6, Hx, Hy = (k2 - k0) h / 4, K = (k2 - k0) t3 / 8, t_ab = (k2 - k0) Pi_ab / 4.
+BTRT_HD void fx_expand3(fx a, fx z, fx X, fx Y, fx Z, fx Hx, fx Hy, fx K, fx txy, fx txz, fx tyz, fx (&r)[19]) {
+    const fx b = fx_ninth(a) >> 1;                // a / 18
+    const fx Hz = -(Hx + Hy), G = (b >> 1) + z - K;
+    r[0] = a - 6 * b - 12 * G;                    // the axis directions sum to 6 b, the diagonals to 12 G
+    const fx bx = b - Hx, by = b - Hy, bz = b - Hz;
+    r[1] = bx + X;
+    r[2] = bx - X;
+    r[3] = by + Y;
+    r[4] = by - Y;
+    r[5] = bz + Z;
+    r[6] = bz - Z;
+    const fx gx = Hx >> 1, gy = Hy >> 1, gz = -(gx + gy);
+    const fx xy = G + gz, xz = G + gy, yz = G + gx;
+    const fx xyp = (X + Y) >> 1, xym = (X - Y) >> 1, xzp = (X + Z) >> 1, xzm = (X - Z) >> 1;
+    const fx yzp = (Y + Z) >> 1, yzm = (Y - Z) >> 1;
+    r[7] = xy - txy + xyp;
+    r[10] = xy - txy - xyp;
+    r[8] = xy + txy - xym;
+    r[9] = xy + txy + xym;
+    r[11] = xz - txz + xzp;
+    r[14] = xz - txz - xzp;
+    r[12] = xz + txz - xzm;
+    r[13] = xz + txz + xzm;
+    r[15] = yz - tyz + yzp;
+    r[18] = yz - tyz - yzp;
+    r[16] = yz + tyz - yzm;
+    r[17] = yz + tyz + yzm;
+}
+
+// Populations of D3Q19 that the FP64 adder converts: 3.45 / 3.29 / 3.27 / 3.51 ms with
+// 0 / 5 / 8 / 12 on the 128^3 hill (20 steps).
+#ifndef BTRT_FX_NADD3
+#define BTRT_FX_NADD3 8
+#endif
+
+// As fx_collide_linear.
+template <bool K0ONE, bool SOURCE>
+BTRT_HD bool fx_collide_linear3(const FxFold3 &q, double (&d)[19], double phi_prev, double src, double &phi_out) {
+    unsigned int em;
+    if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;
+    if (SOURCE && fx_exp(src) > em + (1u << 20)) return false;
+    fx D[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) D[i] = fx_from<kFxTop3>(d[i], em);
+    const FxMoments3 m = fx_moments3(D);
+    const FxArg jx = fx_arg(m.jx), jy = fx_arg(m.jy), jz = fx_arg(m.jz), ph = fx_arg(m.phi);
+    const FxArg pp = fx_arg(fx_from<kFxTop3>(phi_prev, em));
+    FxSum sx = fx_sum(), sy = fx_sum(), sz = fx_sum();
+    fx_add(sx, jx, q.Q[0]);
+    fx_add(sx, jy, q.Q[1]);
+    fx_add(sx, jz, q.Q[2]);
+    fx_add(sx, ph, q.P[0]);
+    fx_add(sx, pp, q.g[0]);
+    fx_add(sy, jx, q.Q[1]);
+    fx_add(sy, jy, q.Q[3]);
+    fx_add(sy, jz, q.Q[4]);
+    fx_add(sy, ph, q.P[1]);
+    fx_add(sy, pp, q.g[1]);
+    fx_add(sz, jx, q.Q[2]);
+    fx_add(sz, jy, q.Q[4]);
+    fx_add(sz, jz, q.Q[5]);
+    fx_add(sz, ph, q.P[2]);
+    fx_add(sz, pp, q.g[2]);
+    fx a = m.phi;
+    if (!K0ONE) a -= 2 * fx_mul(ph, q.om2);
+    if (SOURCE) a += fx_from<kFxTop3>(src, em);
+    fx r[19];
+    fx_expand3(a, 0, fx_value(sx), fx_value(sy), fx_value(sz), fx_mul(fx_arg(m.hx), q.d12), fx_mul(fx_arg(m.hy), q.d12),
+               fx_mul(fx_arg(m.t3), q.d24), fx_mul(fx_arg(m.pxy), q.d4), fx_mul(fx_arg(m.pxz), q.d4),
+               fx_mul(fx_arg(m.pyz), q.d4), r);
+    fx_store<K0ONE, BTRT_FX_NADD3, kFxTop3>(D, r, q.om2, em, d);
+    phi_out = fx_to<kFxTop3>(m.phi, em);
     return true;
 }
 

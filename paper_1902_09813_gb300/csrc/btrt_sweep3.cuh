@@ -51,8 +51,14 @@ template <typename Real> __device__ __forceinline__ Real wgt3(int i) {
     return i == 0 ? cst<Real>(1, 3) : (i <= 6 ? cst<Real>(1, 18) : cst<Real>(1, 36));
 }
 
+// Constants of the integer collision: FP64 lattices only.
+template <typename Real> struct FxPart3 {};
+template <> struct FxPart3<double> {
+    FxFold3 fx;
+};
+
 template <typename Real>
-struct Sweep3Params {
+struct Sweep3Params : FxPart3<Real> {
     const void *fin;       // post-collision populations of the previous step: 19 planes, `plane` apart
     void *fout;
     const Real *phi_in;    // phi of the nodes that wrote fin
@@ -323,6 +329,235 @@ __device__ __forceinline__ Real collide3(const Sweep3Params<Real> &p, Real (&d)[
     return phi;
 }
 
+// ---------------------------------------------------------------- the FP64 collision on the integer pipes
+// As in two dimensions (btrt_fx.cuh, collide_f64): the FP64 forms out of line for
+// the nodes the integer form does not take.  FP64 alone takes 113 operations per node
+// and ran at 0.83 of the FP64 pipe, 4.3 GLUPS at 128^3; with the integer form 13.
+template <int MODE, int SRC>
+static __device__ __noinline__ double collide3_f64_slow(const Sweep3Params<double> &p, double *t, double phi_prev,
+                                                        double srcv) {
+    double d[19], phid;
+#pragma unroll
+    for (int i = 0; i < 19; ++i) d[i] = t[i];
+    const double phi = collide3<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, phid);
+#pragma unroll
+    for (int i = 0; i < 19; ++i) t[i] = d[i];
+    return phi;
+}
+static __device__ __noinline__ void init3_f64_slow(const Sweep3Params<double> &p, double *t, double phi, double src) {
+    double d[19];
+    equilibrium3<double, kShiftNone>(p, phi, d);
+#pragma unroll
+    for (int i = 0; i < 19; ++i) t[i] = fma(wgt3<double>(i), src, d[i]);
+}
+
+__device__ __forceinline__ double reaction3(const Sweep3Params<double> &p, double phi) {
+    return p.react_rate * phi * (1.0 - (p.react2 ? phi * phi : pow_half(phi, p.react_exp, p.re_n, p.re_h)));
+}
+
+// Per-node coefficients or a reaction source: integer moments and populations, FP64
+// coefficients and V.
+template <int MODE, int SRC>
+__device__ __forceinline__ bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19], double phi_prev,
+                                                    double srcv, double &phi_out) {
+    unsigned int em;
+    if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;
+    fx D[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) D[i] = fx_from<kFxTop3>(d[i], em);
+    FxMoments3 m = fx_moments3(D);
+    const double phi = fx_to<kFxTop3>(m.phi, em);
+    fx X, Y, Z, z = 0;
+    FxConst d12, d24, d4;
+    if constexpr (MODE == kGeneral) {
+        const double jx = fx_to<kFxTop3>(m.jx, em), jy = fx_to<kFxTop3>(m.jy, em), jz = fx_to<kFxTop3>(m.jz, em);
+        const double dphi = phi - phi_prev, p2 = phi * phi;
+        double Bx, By, Bz, dBx, dBy, dBz;
+        if (p.bq2) {
+            Bx = fma(p.ux, phi, p.bgx * p2);
+            By = fma(p.uy, phi, p.bgy * p2);
+            Bz = fma(p.uz, phi, p.bgz * p2);
+            const double sp = phi + phi_prev;
+            dBx = fma(p.bgx, sp, p.ux) * dphi;
+            dBy = fma(p.bgy, sp, p.uy) * dphi;
+            dBz = fma(p.bgz, sp, p.uz) * dphi;
+        } else {
+            const double gq = pow_half(phi, p.bq, p.bq_n, p.bq_h);
+            const double dg = gq - pow_half(phi_prev, p.bq, p.bq_n, p.bq_h);
+            Bx = fma(p.ux, phi, p.bgx * gq);
+            By = fma(p.uy, phi, p.bgy * gq);
+            Bz = fma(p.uz, phi, p.bgz * gq);
+            dBx = fma(p.ux, dphi, p.bgx * dg);
+            dBy = fma(p.uy, dphi, p.bgy * dg);
+            dBz = fma(p.uz, dphi, p.bgz * dg);
+        }
+        if (p.c3 != 0.0) {
+            // C(phi) - phi: in 3 t3, and k0 (C - phi) / 24 on the diagonals
+            const double Cm = p.c3 * p2 * phi;
+            if (fx_exp(Cm) > em + (1u << 20)) return false;
+            m.t3 -= fx_from<kFxTop3>(Cm, em);
+            z = fx_from<kFxTop3>(p.k0 * cst<double>(1, 24) * Cm, em);
+        }
+        const double s3 = fma(p.a2x3, p2, 3.0);
+        const double mxx = fma(s3, p.A0[0], 0.5), mxy = s3 * p.A0[1], mxz = s3 * p.A0[2];
+        const double myy = fma(s3, p.A0[3], 0.5), myz = s3 * p.A0[4], mzz = fma(s3, p.A0[5], 0.5);
+        const double cxx = fma(myy, mzz, -(myz * myz)), cxy = fma(mxz, myz, -(mxy * mzz));
+        const double cxz = fma(mxy, myz, -(mxz * myy)), cyy = fma(mxx, mzz, -(mxz * mxz));
+        const double cyz = fma(mxy, mxz, -(mxx * myz)), czz = fma(mxx, myy, -(mxy * mxy));
+        const double det = fma(mxx, cxx, fma(mxy, cxy, mxz * cxz));
+        const double tr = (mxx + myy) + mzz;
+        double id, k2;
+        if (p.k2_hbb) {
+            const double q2 = fma(4.0, tr, -3.0);
+            const double rc = recip_f64(det * q2);
+            id = rc * q2;
+            k2 = (fma(cst<double>(16, 3), tr, -8.0) * det) * rc;
+        } else {
+            id = recip_f64(det);
+            k2 = p.k2c;
+        }
+        const double dk = k2 - p.k0;
+        // K1 e with the cofactors, divided by the determinant once per component
+        const double ex = id * fma(-0.5, dBx, Bx - jx), ey = id * fma(-0.5, dBy, By - jy), ez = id * fma(-0.5, dBz, Bz - jz);
+        const double Vx = fma(cxx, ex, fma(cxy, ey, fma(cxz, ez, fma(p.k0, jx, dBx))));
+        const double Vy = fma(cxy, ex, fma(cyy, ey, fma(cyz, ez, fma(p.k0, jy, dBy))));
+        const double Vz = fma(cxz, ex, fma(cyz, ey, fma(czz, ez, fma(p.k0, jz, dBz))));
+        const unsigned int far = em + (2u << 20);
+        if (fx_exp(dk) > (1023u << 20) || fx_exp(Vx) > far || fx_exp(Vy) > far || fx_exp(Vz) > far) return false;
+        const FxConst sixth = {0x2aaaaaab, (int)0xaaaaaaab};   // 2^64 / 6
+        X = fx_mul(fx_arg(fx_from<kFxTop3>(Vx, em)), sixth);
+        Y = fx_mul(fx_arg(fx_from<kFxTop3>(Vy, em)), sixth);
+        Z = fx_mul(fx_arg(fx_from<kFxTop3>(Vz, em)), sixth);
+        const FxArg c = fx_arg(fx_from(dk, 1019u << 20));      // dk / 4 in units of 2^-64
+        d4.hi = c.h;
+        d4.lo = c.l;
+        d12 = d24 = d4;
+        // (k2 - k0)/12 and /24 as (k2 - k0)/4 of a third and a sixth of the moment
+        m.hx = 2 * fx_mul(fx_arg(m.hx), sixth);
+        m.hy = 2 * fx_mul(fx_arg(m.hy), sixth);
+        m.t3 = fx_mul(fx_arg(m.t3), sixth);
+    } else {
+        const FxArg jx = fx_arg(m.jx), jy = fx_arg(m.jy), jz = fx_arg(m.jz), ph = fx_arg(m.phi);
+        const FxArg pp = fx_arg(fx_from<kFxTop3>(phi_prev, em));
+        FxSum s[3] = {fx_sum(), fx_sum(), fx_sum()};
+        constexpr int at[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            fx_add(s[a], jx, p.fx.Q[at[a][0]]);
+            fx_add(s[a], jy, p.fx.Q[at[a][1]]);
+            fx_add(s[a], jz, p.fx.Q[at[a][2]]);
+            fx_add(s[a], ph, p.fx.P[a]);
+            fx_add(s[a], pp, p.fx.g[a]);
+        }
+        X = fx_value(s[0]);
+        Y = fx_value(s[1]);
+        Z = fx_value(s[2]);
+        d12 = p.fx.d12;
+        d24 = p.fx.d24;
+        d4 = p.fx.d4;
+    }
+    double src = 0.0;
+    if constexpr (SRC == kSrcReaction) srcv = fma(1.5, reaction3(p, phi), -0.5 * reaction3(p, phi_prev));
+    if constexpr (SRC != kSrcNone) src = p.src_val * srcv;
+    if (SRC != kSrcNone && fx_exp(src) > em + (1u << 20)) return false;
+    const bool k0_one = MODE == kLinearK0One || p.k0_one;
+    fx a = m.phi, r[19];
+    if (!k0_one) a -= 2 * fx_mul(fx_arg(m.phi), p.fx.om2);
+    if (SRC != kSrcNone) a += fx_from<kFxTop3>(src, em);
+    fx_expand3(a, z, X, Y, Z, fx_mul(fx_arg(m.hx), d12), fx_mul(fx_arg(m.hy), d12), fx_mul(fx_arg(m.t3), d24),
+               fx_mul(fx_arg(m.pxy), d4), fx_mul(fx_arg(m.pxz), d4), fx_mul(fx_arg(m.pyz), d4), r);
+    if (k0_one) fx_store<true, 0, kFxTop3>(D, r, p.fx.om2, em, d);
+    else fx_store<false, 0, kFxTop3>(D, r, p.fx.om2, em, d);
+    phi_out = phi;
+    return true;
+}
+
+// The initialising collision: f^eq + w S (init_f64 in three dimensions).
+template <int MODE, int SRC>
+__device__ __forceinline__ void init3_f64(const Sweep3Params<double> &p, double (&d)[19], double phi, double src) {
+    double Bx = p.ux * phi, By = p.uy * phi, Bz = p.uz * phi, Cm = 0.0;
+    if constexpr (MODE == kGeneral) {
+        const double g = p.bq2 ? phi * phi : pow_half(phi, p.bq, p.bq_n, p.bq_h);
+        Bx = fma(p.bgx, g, Bx);
+        By = fma(p.bgy, g, By);
+        Bz = fma(p.bgz, g, Bz);
+        Cm = p.c3 * phi * phi * phi;
+    }
+    unsigned int em = fx_exp(phi);
+    em = em > kFxExpMin ? em : kFxExpMin;
+    const unsigned int far = em + (1u << 20);
+    if (em > kFxExpMax || fx_exp(Bx) > far || fx_exp(By) > far || fx_exp(Bz) > far || fx_exp(src) > far ||
+        fx_exp(Cm) > far) {
+        double t[19];
+        init3_f64_slow(p, t, phi, src);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) d[i] = t[i];
+        return;
+    }
+    const FxConst sixth = {0x2aaaaaab, (int)0xaaaaaaab};   // 2^64 / 6
+    fx a = fx_from<kFxTop3>(phi, em), z = 0, r[19];
+    if (SRC != kSrcNone) a += fx_from<kFxTop3>(src, em);
+    if (MODE == kGeneral) z = fx_from<kFxTop3>(cst<double>(1, 24) * Cm, em);
+    fx_expand3(a, z, fx_mul(fx_arg(fx_from<kFxTop3>(Bx, em)), sixth),
+               fx_mul(fx_arg(fx_from<kFxTop3>(By, em)), sixth),
+               fx_mul(fx_arg(fx_from<kFxTop3>(Bz, em)), sixth), 0, 0, 0, 0, 0, 0, r);
+    fx_store<true, BTRT_FX_NADD3, kFxTop3>(r, r, p.fx.om2, em, d);
+}
+
+template <int MODE, int SRC>
+__device__ __forceinline__ double collide3_f64(const Sweep3Params<double> &p, double (&d)[19], double phi_prev,
+                                               double srcv) {
+    if (p.first) {
+        init3_f64<MODE, SRC>(p, d, phi_prev, SRC == kSrcReaction ? p.src_val * reaction3(p, phi_prev)
+                                             : SRC != kSrcNone   ? p.src_val * srcv
+                                                                 : 0.0);
+        return phi_prev;
+    }
+    double phi;
+    bool done = false;
+    if (p.fx.ok & (MODE == kGeneral ? kFxOkGeneral : kFxOkLinear)) {
+        if constexpr (MODE == kGeneral || SRC == kSrcReaction)
+            done = fx_collide_general3<MODE, SRC>(p, d, phi_prev, srcv, phi);
+        else
+            done = fx_collide_linear3<MODE == kLinearK0One, SRC != kSrcNone>(
+                p.fx, d, phi_prev, SRC != kSrcNone ? p.src_val * srcv : 0.0, phi);
+    }
+    if (!done) {
+        double t[19];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) t[i] = d[i];
+        phi = collide3_f64_slow<MODE, SRC>(p, t, phi_prev, srcv);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) d[i] = t[i];
+    }
+    return phi;
+}
+
+// Element `at` of population plane i: the plane's base is uniform over the launch and
+// the byte offset in it fits 32 bits (see plane_at).
+__device__ __forceinline__ const double *plane3_f64(const Sweep3Params<double> &p, const double *f, int i, int at) {
+#ifdef BTRT_DEBUG_BOUNDS
+    return f + BTRT_IX(p.flags, i * p.plane + at, 19 * p.plane);
+#else
+    return reinterpret_cast<const double *>(reinterpret_cast<const char *>(f + (size_t)i * p.plane) + (unsigned int)at * 8u);
+#endif
+}
+
+// Resident blocks per SM asked of the compiler (0: its choice).
+// FP64, 128^3 hill, 20 steps: three blocks (80 registers) 3.27 ms, two 3.72, four 3.31,
+// five 4.09; per-node coefficients three (80 registers, spilling) 8.14 against 8.44 with
+// two (128) and 11.5 with one.
+#ifndef BTRT3_MINBLOCKS_F64
+#define BTRT3_MINBLOCKS_F64 3
+#endif
+#ifndef BTRT3_MINBLOCKS_F64_GEN
+#define BTRT3_MINBLOCKS_F64_GEN 3
+#endif
+template <typename Real, int MODE, int SRC> struct MinBlocks3 { static constexpr int value = 0; };
+template <int MODE, int SRC> struct MinBlocks3<double, MODE, SRC> {
+    static constexpr int value = MODE == kLinearK0One && SRC != kSrcReaction ? BTRT3_MINBLOCKS_F64 : BTRT3_MINBLOCKS_F64_GEN;
+};
+
 // Pull of a node with at least one neighbour across the domain boundary.
 template <typename Real, typename S, int SH>
 __device__ __forceinline__ void pull3_boundary(const Sweep3Params<Real> &p, const S *__restrict__ fin, int x, int y,
@@ -357,7 +592,7 @@ __device__ __forceinline__ void pull3_boundary(const Sweep3Params<Real> &p, cons
 }
 
 template <typename Real, typename S, int SH, int MODE, int SRC>
-__global__ void __launch_bounds__(256) sweep3_kernel(const __grid_constant__ Sweep3Params<Real> p) {
+__global__ void __launch_bounds__(256, MinBlocks3<Real, MODE, SRC>::value) sweep3_kernel(const __grid_constant__ Sweep3Params<Real> p) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -367,13 +602,17 @@ __global__ void __launch_bounds__(256) sweep3_kernel(const __grid_constant__ Swe
     const int node = z * p.slab + y * p.pitch + x;
     const Real phi_prev = p.phi_in[BTRT_IX(p.flags, node, p.plane)];
     Real d[19];
-    if (p.first) {
-        equilibrium3<Real, SH>(p, phi_prev, d);
+    if (p.first) {   // FP64: formed in the collision (init3_f64)
+        if constexpr (!std::is_same<Real, double>::value) equilibrium3<Real, SH>(p, phi_prev, d);
     } else if (x > 0 && x < p.nx - 1 && y > 0 && y < p.ny - 1 && z > 0 && z < p.nz - 1) {
 #pragma unroll
-        for (int i = 0; i < 19; ++i)
-            d[i] = Storage<S>::load(
-                fin[BTRT_IX(p.flags, i * p.plane + node - cz3(i) * p.slab - cy3(i) * p.pitch - cx3(i), 19 * p.plane)]);
+        for (int i = 0; i < 19; ++i) {
+            if constexpr (std::is_same<Real, double>::value)
+                d[i] = *plane3_f64(p, fin, i, node - cz3(i) * p.slab - cy3(i) * p.pitch - cx3(i));
+            else
+                d[i] = Storage<S>::load(
+                    fin[BTRT_IX(p.flags, i * p.plane + node - cz3(i) * p.slab - cy3(i) * p.pitch - cx3(i), 19 * p.plane)]);
+        }
         if constexpr (SH == kShiftLocal) {
 #pragma unroll
             for (int i = 1; i < 19; ++i)
@@ -389,13 +628,19 @@ __global__ void __launch_bounds__(256) sweep3_kernel(const __grid_constant__ Swe
     if constexpr (SRC == kSrcConst) srcv = Real(1);
     if constexpr (SRC == kSrcField) srcv = p.srcF[BTRT_IX(p.flags, node, p.plane)];
     const Real rs = SH == kShiftLocal ? phi_prev : p.phi_ref;
-    Real phid;
-    const Real phi = collide3<Real, MODE, SRC, SH>(p, d, rs, phi_prev, srcv, p.first != 0, phid);
+    Real phid, phi;
+    if constexpr (std::is_same<Real, double>::value) {
+        phi = collide3_f64<MODE, SRC>(p, d, phi_prev, srcv);
+        phid = phi;
+    } else {
+        phi = collide3<Real, MODE, SRC, SH>(p, d, rs, phi_prev, srcv, p.first != 0, phid);
+    }
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
         Real v = d[i];
         if constexpr (SH == kShiftLocal) v = fma(-wgt3<Real>(i), phid, v);
-        fout[BTRT_IX(p.flags, i * p.plane + node, 19 * p.plane)] = Storage<S>::pack(v);
+        if constexpr (std::is_same<Real, double>::value) *const_cast<double *>(plane3_f64(p, fout, i, node)) = v;
+        else fout[BTRT_IX(p.flags, i * p.plane + node, 19 * p.plane)] = Storage<S>::pack(v);
     }
     p.phi_out[BTRT_IX(p.flags, node, p.plane)] = phi;
     if (not_finite(phi)) atomicOr(p.flags, 1);
