@@ -91,7 +91,7 @@ FP64_NOMINAL_TOPS = 0.625
 # to them both are re-taken and the digest updated (a CPU test checks it), and
 # until then the traffic is reported as null.
 FP64_SWEEP_SOURCES = ("btrt_sweep.cuh", "btrt_dw.cuh", "btrt_fx.cuh")   # the FP64 sweep's device code
-FP64_SWEEP_DIGEST = "0db4295df9ce7ce1"
+FP64_SWEEP_DIGEST = "7da734b66b7bcd4f"
 FP64_TRAFFIC_PER_NODE = 148.4
 # DRAM bytes per node and step of the two-step FP32-compute kernel measured by ncu,
 # keyed by (storage, shift), for the sources with digest TB2_DIGEST.
@@ -135,11 +135,21 @@ def measure_fp64_peak(iters: int = 2000):
             "kernel": "fp64_chains (4/8/16 independent chains per thread, whole waves, best per kind)"}
 
 
+def many_steps_form(args) -> bool:
+    """Small lattices: many steps per launch (the library's takes_tbn)."""
+    general = args.workload != "mms"
+    most = {"f64": 3 << 13 if general else 1 << 15, "df64": 1 << 15 if general else 1 << 16}.get(
+        args.compute, 1 << 17 if args.storage == "f32" and args.shift not in ("local_dw", "local_dw_sr") else 1 << 18)
+    return 32 <= args.n and args.n * args.n <= most
+
+
 def kernel_form(args) -> str:
     """The kernel form of the timed steps: what the library's AUTO resolves to for
     FP32 compute (the vector form for FP16/BF16 storage on lattices of 2^21 nodes
     or more, two steps per launch otherwise), the form asked for, or the plain
     sweep."""
+    if args.sweep == "auto" and many_steps_form(args):
+        return "tbn"
     if args.compute != "f32" or args.shift in ("local_dw", "local_dw_sr"):
         return "plain"
     if args.sweep != "auto":
@@ -397,7 +407,8 @@ def run_gpu(args):
                 "h2d_bytes_per_step": int(8 * nodes / args.steps),
                 "d2h_bytes_per_step": int(8 * nodes / args.steps),
                 "note": "one solve per K steps: phi0 in, phi out, amortised per step"},
-            "gpu_launches": (args.steps // 2 + args.steps % 2) if two_step_form(args) else args.steps,
+            "gpu_launches": (args.steps // 2 + args.steps % 2) if two_step_form(args)
+            else -(-args.steps // 256) if kernel_form(args) == "tbn" else args.steps,
             "clocks": clk,
         }
         line.update(extra)

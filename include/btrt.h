@@ -207,11 +207,12 @@ btrt_status btrt_mass(btrt_lattice L, double *out);
 
 /* Flags raised by the sweep since the last btrt_init_phi: bit 0 = some node
  * produced a NaN/Inf phi (returns BTRT_EUNSTABLE), bit 2 = a bounded wait for a
- * tile copy gave up (returns BTRT_ETIMEOUT), bit 3 = an index check of a
+ * tile copy or at a grid barrier gave up (returns BTRT_ETIMEOUT), bit 3 = an index check of a
  * -DBTRT_DEBUG_BOUNDS build failed (returns BTRT_ECUDA).  Synchronises. */
 btrt_status btrt_check(btrt_lattice L, int32_t *flags);
 
-/* Kernel form of the ordinary FP32-compute sweep: BTRT_SWEEP_AUTO (default: the
+/* Kernel form of the ordinary FP32-compute sweep: BTRT_SWEEP_AUTO (default: small
+ * lattices advance up to 256 steps in one cooperative launch, in every format; the
  * faster form as measured on GB300: BTRT_SWEEP_VEC for F16/BF16 storage on
  * lattices of 2^21 nodes or more, BTRT_SWEEP_TB2 otherwise), BTRT_SWEEP_PLAIN
  * (one step per launch, direct global loads served by L1/L2), BTRT_SWEEP_TMA
@@ -227,7 +228,7 @@ btrt_status btrt_check(btrt_lattice L, int32_t *flags);
  * vector access of BTRT_SWEEP_VEC in both steps and the intermediate step kept
  * in shared memory in the storage format).  Every storage format and shift of
  * an FP32-compute lattice.  All forms give bitwise identical results.  FP64 and
- * double-word lattices always use the plain form (BTRT_SWEEP_TMA, _TB2, _VEC and
+ * double-word lattices use the plain form or, small, AUTO's (BTRT_SWEEP_TMA, _TB2, _VEC and
  * _TB2V: BTRT_EINVAL). */
 enum {
     BTRT_SWEEP_AUTO = 0, BTRT_SWEEP_PLAIN = 1, BTRT_SWEEP_TMA = 2, BTRT_SWEEP_TB2 = 3, BTRT_SWEEP_VEC = 4,

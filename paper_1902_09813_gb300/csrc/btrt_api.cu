@@ -20,6 +20,7 @@
 
 #include "../../include/btrt.h"
 #include "btrt_internal.h"
+#include "btrt_tbn.cuh"
 
 #include <cudaTypedefs.h>
 
@@ -152,7 +153,7 @@ Layout make_layout(const btrt_grid_desc *g) {
     L.off_wall = off;
     off += align_up(4 * (size_t)L.maxside * sr, kAlign);
     L.off_red = off;
-    off += align_up((kRedBlocks + 2) * sizeof(double) + 16, kAlign);
+    off += align_up((kRedBlocks + 2) * sizeof(double) + 16 + 16, kAlign);   // partials, sum, flags, barrier
     L.resid_blocks = sweep_blocks(g->nx, g->ny, g->compute, g->storage);
     L.off_resid = off;
     off += align_up((size_t)L.resid_blocks * sizeof(double), kAlign);
@@ -415,7 +416,8 @@ int btrt::sweep_mode(btrt_lattice L) {
 // steps each, one after the other: 10.5 s with the vector form, 6.8 s with two
 // steps per launch).
 // Stochastically rounded storage has the plain and vector forms only: the vector
-// form from kVecAutoNodes on, the plain one below.
+// form from kVecAutoNodes on, the plain one below.  btrt_step takes small lattices
+// many steps per launch before it asks for this form (takes_tbn).
 constexpr long long kVecAutoNodes = 1LL << 21;
 int btrt::effective_sweep_variant(btrt_lattice L) {
     if (L->g.compute != BTRT_F32 || has_phi_lo(L->g)) return BTRT_SWEEP_PLAIN;
@@ -452,6 +454,53 @@ btrt_status launch(btrt_lattice L, int64_t n, bool first, bool resid = false) {
         else
             CUDA_TRY(launch_sweep_f32(p, L->g.storage, sh, sweep_mode(L), L->stream));
     }
+    return BTRT_OK;
+}
+
+// Whether btrt_step advances L many steps per launch (btrt_tbn.cuh): AUTO, sides of at
+// least one region width, and few enough nodes.  Measured us per step, many steps per
+// launch against the form AUTO takes otherwise (square lattices, 200 steps with set-up
+// and read): FP32 storage 64^2 1.7 / 5.2, 256^2 2.6 / 5.2, 362^2 3.8 / 5.3, 430^2 5.7 / 5.3;
+// FP16 local shift 64^2 1.8 / 6.3, 362^2 3.9 / 6.3, 512^2 6.5 / 7.3 (nonlinear 6.8 / 9.4);
+// double-word phi 512^2 7.1 / 10.4, first-moment form 8.3 / 10.4; FP64 hill 64^2 2.1 / 6.3,
+// 160^2 3.1 / 6.3, 181^2 5.0 / 6.3, 256^2 6.9 / 6.3, nonlinear 160^2 10.2 / 12.3, 181^2
+// 14.8 / 12.4; double-word format hill 256^2 6.1 / 6.3, nonlinear 181^2 6.2 / 6.3.
+bool takes_tbn(btrt_lattice L) {
+    const btrt_grid_desc &g = L->g;
+    if (L->sweep_variant != BTRT_SWEEP_AUTO || g.nx < 32 || g.ny < 32) return false;
+    const bool general = sweep_mode(L) == kGeneral;
+    long long most;
+    if (g.compute == BTRT_F64) most = general ? 3 << 13 : 1 << 15;
+    else if (g.compute == BTRT_DF64) most = general ? 1 << 15 : 1 << 16;
+    else if (g.storage == BTRT_F32 && !has_phi_lo(g)) most = 1 << 17;
+    else most = 1 << 18;
+    return (long long)g.nx * g.ny <= most;
+}
+
+template <typename Real>
+btrt_status launch_tbn(btrt_lattice L, int n) {
+    SweepParams<Real> p;
+    fill_params(L, p, L->step + 1, false);
+    TbnSteps<Real> st;
+    st.n = n;
+    st.step0 = L->step + 1;
+    st.barrier = L->barrier();
+    st.wait_limit = 1ull << 22;
+    for (int k = 0; k < n; ++k) {
+        double sv = 0.0, wf = 1.0;
+        step_scalars(L, L->step + 1 + k, false, &sv, &wf);
+        st.src_val[k] = (Real)sv;
+        st.wall_fac[k] = (Real)wf;
+    }
+    const int mode = sweep_mode(L), sh = shift_of(L->g);
+    int rounds = 0;   // one buffer flip each
+    if constexpr (std::is_same<Real, double>::value) CUDA_TRY(launch_sweep_tbn_f64(p, st, mode, &rounds, L->stream));
+    else if constexpr (std::is_same<Real, dw>::value) CUDA_TRY(launch_sweep_tbn_dw(p, st, mode, &rounds, L->stream));
+    else if (L->g.storage == BTRT_F32) CUDA_TRY(launch_sweep_tbn_f32(p, st, sh, mode, &rounds, L->stream));
+    else if (L->g.storage == BTRT_F16) CUDA_TRY(launch_sweep_tbn_f16(p, st, sh, mode, &rounds, L->stream));
+    else CUDA_TRY(launch_sweep_tbn_bf16(p, st, sh, mode, &rounds, L->stream));
+    L->cur = (L->cur + rounds) & 1;
+    L->step += n;
     return BTRT_OK;
 }
 
@@ -808,6 +857,15 @@ btrt_status btrt_step(btrt_lattice L, int64_t nsteps) {
     if (!L) return fail(BTRT_EINVAL, "null lattice");
     if (!L->ready) return fail(BTRT_ESTATE, "lattice not initialised");
     if (nsteps < 0) return fail(BTRT_EINVAL, "negative step count");
+    if (takes_tbn(L))
+        while (nsteps >= 2) {
+            const int n = (int)std::min<int64_t>(nsteps, kTbnMaxSteps);
+            btrt_status st = L->g.compute == BTRT_F64    ? launch_tbn<double>(L, n)
+                             : L->g.compute == BTRT_DF64 ? launch_tbn<dw>(L, n)
+                                                         : launch_tbn<float>(L, n);
+            if (st != BTRT_OK) return st;
+            nsteps -= n;
+        }
     // the two-step forms serve every FP32-compute lattice (AUTO: see effective_sweep_variant)
     const int form = effective_sweep_variant(L);
     if (form == BTRT_SWEEP_TB2 || form == BTRT_SWEEP_TB2V) {
@@ -952,7 +1010,7 @@ btrt_status btrt_check(btrt_lattice L, int32_t *flags) {
     CUDA_TRY(cudaMemcpyAsync(flags, L->flags(), sizeof(int32_t), cudaMemcpyDeviceToHost, L->stream));
     CUDA_TRY(cudaStreamSynchronize(L->stream));
     if (*flags & 8) return fail(BTRT_ECUDA, "an index check of the debug build failed (flag bit 3)");
-    if (*flags & 4) return fail(BTRT_ETIMEOUT, "a bounded wait for a tile copy gave up");
+    if (*flags & 4) return fail(BTRT_ETIMEOUT, "a bounded wait (tile copy or grid barrier) gave up");
     if (*flags & 1) return fail(BTRT_EUNSTABLE, "non-finite phi detected (unstable parameters?)");
     return BTRT_OK;
 }

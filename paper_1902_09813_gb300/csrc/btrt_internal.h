@@ -42,17 +42,6 @@ inline bool stochastic_store(const btrt_grid_desc &g) {
 // after the phi plane of each buffer).
 inline bool has_j(const btrt_grid_desc &g) { return g.shift == BTRT_SHIFT_MOMENT_SR; }
 
-// Stochastic-rounding seed of the step that produces step index n: the SplitMix64
-// output function (Steele, Lea and Flood, 2014) of the step index.  Host and
-// device (the batch kernels derive each step's seed from the member's step count)
-// compute the same value.
-__host__ __device__ inline unsigned int sr_step_seed(long long n) {
-    unsigned long long z = (unsigned long long)n * 0x9e3779b97f4a7c15ull + 0x632be59bd9b4e019ull;
-    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-    return (unsigned int)(z ^ (z >> 31));
-}
-
 }  // namespace btrt
 
 // The host-side lattice object behind btrt_lattice.
@@ -102,6 +91,8 @@ struct btrt_lattice_s {
     template <typename Real> Real *af() { return lay.off_af ? reinterpret_cast<Real *>(ws + lay.off_af) : nullptr; }
     double *red_out() { return partials() + btrt::kRedBlocks; }
     int *flags() { return reinterpret_cast<int *>(partials() + btrt::kRedBlocks + 2); }
+    // arrivals at the grid barrier of many steps per launch (in the region's padding)
+    unsigned int *barrier() { return reinterpret_cast<unsigned int *>(flags() + 4); }
 };
 
 namespace btrt {
@@ -179,6 +170,20 @@ cudaError_t launch_sweep_tb2v_f16(const SweepParams<float> &pa, const SweepParam
                                   cudaStream_t s);
 cudaError_t launch_sweep_tb2v_bf16(const SweepParams<float> &pa, const SweepParams<float> &pb, int shift, int mode,
                                    cudaStream_t s);
+
+// Many steps per launch (btrt_tbn.cuh): p holds the parameters of the first step, its
+// buffers in fin, phi_in and the others in fout, phi_out; *rounds: buffer flips.
+template <typename Real> struct TbnSteps;
+cudaError_t launch_sweep_tbn_f64(const SweepParams<double> &p, TbnSteps<double> &st, int mode, int *rounds,
+                                 cudaStream_t s);
+cudaError_t launch_sweep_tbn_dw(const SweepParams<dw> &p, TbnSteps<dw> &st, int mode, int *rounds,
+                                 cudaStream_t s);
+cudaError_t launch_sweep_tbn_f32(const SweepParams<float> &p, TbnSteps<float> &st, int shift, int mode, int *rounds,
+                                 cudaStream_t s);
+cudaError_t launch_sweep_tbn_f16(const SweepParams<float> &p, TbnSteps<float> &st, int shift, int mode, int *rounds,
+                                 cudaStream_t s);
+cudaError_t launch_sweep_tbn_bf16(const SweepParams<float> &p, TbnSteps<float> &st, int shift, int mode, int *rounds,
+                                 cudaStream_t s);
 
 // One step per launch with vector memory access (FP32 compute; storage BTRT_F32,
 // F16 or BF16; shift kShiftRef or kShiftLocal); never the initialising collision

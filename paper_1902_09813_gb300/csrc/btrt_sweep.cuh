@@ -313,7 +313,8 @@ constexpr int kFp64OpsPerNodeLinearTrig = 50;
 template <typename Real, int MODE, int SRC, int SH>
 __device__ __forceinline__ Real collide_fold(const SweepParams<Real> &p, Real (&d)[9], Real rs, Real phi_prev,
                                              Real srcv, bool first, int node, Real &phid_out,
-                                             const FoldConsts<Real> *Lc = nullptr) {
+                                             const FoldConsts<Real> *Lc = nullptr, const Real *sv = nullptr) {
+    const Real src_val = sv ? *sv : p.src_val;   // the step's source factor (several steps per launch: its own)
     // the folded constants: p.lin, or the copy at Lc (a batch keeps its members'
     // copies in the kernel's parameter space)
     const FoldConsts<Real> &L = Lc ? *Lc : p.lin;
@@ -426,7 +427,7 @@ __device__ __forceinline__ Real collide_fold(const SweepParams<Real> &p, Real (&
             srcv = fma(Real(1.5), Sn, Real(-0.5) * Sp);
         }
     }
-    if constexpr (SRC != 0) a = fma(p.src_val, srcv, a);
+    if constexpr (SRC != 0) a = fma(src_val, srcv, a);
     const Real w0 = cst<Real>(4, 9), w1 = cst<Real>(1, 9), w5 = cst<Real>(1, 36);
     const Real v1 = cst<Real>(1, 3), v5 = cst<Real>(1, 12);   // 3 w1, 3 w5
     Real r[9];
@@ -470,11 +471,12 @@ __device__ __forceinline__ Real collide_fold(const SweepParams<Real> &p, Real (&
 // the integer form does not take, and the initialising collision.
 template <int MODE, int SRC>
 static __device__ __noinline__ double collide_f64_slow(const SweepParams<double> &p, double *t, double phi_prev,
-                                                       double srcv, int node) {
+                                                       double srcv, int node, double src_val) {
     double d[9], phid;
 #pragma unroll
     for (int i = 0; i < 9; ++i) d[i] = t[i];
-    const double phi = collide_fold<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, node, phid);
+    const double phi = collide_fold<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, node, phid,
+                                                                     nullptr, &src_val);
 #pragma unroll
     for (int i = 0; i < 9; ++i) t[i] = d[i];
     return phi;
@@ -497,7 +499,7 @@ __device__ __forceinline__ double recip_f64(double v) {
 // the integer form's range.
 template <int MODE, int SRC>
 __device__ __forceinline__ bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], double phi_prev,
-                                                   double srcv, int node, double &phi_out) {
+                                                   double srcv, int node, double src_val, double &phi_out) {
     const FoldConsts<double> &L = p.lin;
     unsigned int em;
     if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;
@@ -590,7 +592,7 @@ __device__ __forceinline__ bool fx_collide_general(const SweepParams<double> &p,
         if (SRC == kSrcReaction || p.src_kind == kSrcReaction)
             srcv = fma(1.5, reaction(p, phi), -0.5 * reaction(p, phi_prev));
     }
-    if constexpr (SRC != kSrcNone) src = p.src_val * srcv;
+    if constexpr (SRC != kSrcNone) src = src_val * srcv;
     if (SRC != kSrcNone && fx_exp(src) > em + (1u << 20)) return false;
     const fx ks = fx_mul(fx_arg(m.s32), d18), t1 = fx_mul(fx_arg(m.del), d4), t5 = fx_mul(fx_arg(m.pxy), d4);
     fx a = m.phi, r[9];
@@ -647,11 +649,11 @@ __device__ __forceinline__ void init_f64(const SweepParams<double> &p, double (&
 // 37 GLUPS (0.89 of HBM) and 10.8.
 template <int MODE, int SRC>
 __device__ __forceinline__ double collide_f64(const SweepParams<double> &p, double (&d)[9], double phi_prev,
-                                              double srcv, int node) {
+                                              double srcv, int node, double src_val) {
     constexpr bool LATE = SRC == kSrcReaction || SRC == kSrcRuntime;   // the source may depend on phi
     if (p.first) {
-        double src = SRC != kSrcNone ? p.src_val * srcv : 0.0;
-        if (LATE && (SRC == kSrcReaction || p.src_kind == kSrcReaction)) src = p.src_val * reaction(p, phi_prev);
+        double src = SRC != kSrcNone ? src_val * srcv : 0.0;
+        if (LATE && (SRC == kSrcReaction || p.src_kind == kSrcReaction)) src = src_val * reaction(p, phi_prev);
         init_f64<MODE, SRC>(p, d, phi_prev, src);
         return phi_prev;
     }
@@ -659,17 +661,17 @@ __device__ __forceinline__ double collide_f64(const SweepParams<double> &p, doub
     bool done = false;
     if (p.fx.ok & (MODE == kGeneral ? kFxOkGeneral : kFxOkLinear)) {
         if constexpr (MODE == kGeneral || LATE)
-            done = fx_collide_general<MODE, SRC>(p, d, phi_prev, srcv, node, phi);
+            done = fx_collide_general<MODE, SRC>(p, d, phi_prev, srcv, node, src_val, phi);
         else if (MODE == kLinearK0One || p.k0_one)
-            done = fx_collide_linear<true, SRC != kSrcNone>(p.fx, d, phi_prev, SRC != kSrcNone ? p.src_val * srcv : 0.0, phi);
+            done = fx_collide_linear<true, SRC != kSrcNone>(p.fx, d, phi_prev, SRC != kSrcNone ? src_val * srcv : 0.0, phi);
         else
-            done = fx_collide_linear<false, SRC != kSrcNone>(p.fx, d, phi_prev, SRC != kSrcNone ? p.src_val * srcv : 0.0, phi);
+            done = fx_collide_linear<false, SRC != kSrcNone>(p.fx, d, phi_prev, SRC != kSrcNone ? src_val * srcv : 0.0, phi);
     }
     if (!done) {
         double t[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) t[i] = d[i];
-        phi = collide_f64_slow<MODE, SRC>(p, t, phi_prev, srcv, node);
+        phi = collide_f64_slow<MODE, SRC>(p, t, phi_prev, srcv, node, src_val);
 #pragma unroll
         for (int i = 0; i < 9; ++i) d[i] = t[i];
     }
@@ -732,6 +734,16 @@ __device__ __forceinline__ bool not_finite(float v) {
 // odd constant (the product's high bits are used).  They depend only on the
 // node, the step index and the population, so every kernel form stores the same
 // values.
+// Stochastic-rounding seed of the step that produces step index n: the SplitMix64
+// output function (Steele, Lea and Flood, 2014) of the step index.  Host and
+// device (the batch kernels derive each step's seed from the member's step count)
+// compute the same value.
+__host__ __device__ inline unsigned int sr_step_seed(long long n) {
+    unsigned long long z = (unsigned long long)n * 0x9e3779b97f4a7c15ull + 0x632be59bd9b4e019ull;
+    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+    return (unsigned int)(z ^ (z >> 31));
+}
 __device__ __forceinline__ unsigned int sr_node_bits(unsigned int seed, int node) {
     unsigned int h = (unsigned int)node ^ seed;
     h ^= h >> 16;
@@ -1081,7 +1093,7 @@ __device__ __forceinline__ double finish_node(const SweepParams<Real> &p, int x,
     const Real rs = SC == kShiftLocal ? phi_prev : p.phi_ref;
     Real phid, phi;
     if constexpr (std::is_same<Real, double>::value) {
-        phi = collide_f64<MODE, SRC>(p, f, phi_prev, src, node);
+        phi = collide_f64<MODE, SRC>(p, f, phi_prev, src, node, p.src_val);
         phid = phi;
     } else {
         phi = collide_fold<Real, MODE, SRC, SC>(p, f, rs, phi_prev, src, p.first != 0, node, phid, Lc);
