@@ -33,6 +33,29 @@ inline cudaError_t launch3_mode(const Sweep3Params<Real> &p, int mode, cudaStrea
     return cudaGetLastError();
 }
 
+// Two nodes per thread: 32 x 8 threads, 64 x 8 nodes per block.
+template <typename S, int SH, int MODE>
+inline void launch3_vec_src(const Sweep3Params<float> &p, cudaStream_t s) {
+    const dim3 g = sweep3_grid((p.nx + 1) / 2, p.ny, p.nz), b = sweep3_block();
+    switch (p.src_kind) {
+    case kSrcNone: sweep3_vec_kernel<S, SH, MODE, kSrcNone><<<g, b, 0, s>>>(p); break;
+    case kSrcConst: sweep3_vec_kernel<S, SH, MODE, kSrcConst><<<g, b, 0, s>>>(p); break;
+    case kSrcField: sweep3_vec_kernel<S, SH, MODE, kSrcField><<<g, b, 0, s>>>(p); break;
+    default: sweep3_vec_kernel<S, SH, MODE, kSrcReaction><<<g, b, 0, s>>>(p); break;
+    }
+}
+template <typename S>
+inline cudaError_t launch3_vec(const Sweep3Params<float> &p, int shift, int mode, cudaStream_t s) {
+    if (shift == kShiftLocal) {
+        if (mode == kLinearK0One) launch3_vec_src<S, kShiftLocal, kLinearK0One>(p, s);
+        else launch3_vec_src<S, kShiftLocal, kLinear>(p, s);
+    } else {
+        if (mode == kLinearK0One) launch3_vec_src<S, kShiftRef, kLinearK0One>(p, s);
+        else launch3_vec_src<S, kShiftRef, kLinear>(p, s);
+    }
+    return cudaGetLastError();
+}
+
 template <typename S>
 inline cudaError_t launch3_f32_storage(const Sweep3Params<float> &p, int shift, int mode, cudaStream_t s) {
     return shift == kShiftLocal ? launch3_mode<float, S, kShiftLocal>(p, mode, s)

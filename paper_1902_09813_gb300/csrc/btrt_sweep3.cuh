@@ -686,4 +686,120 @@ __global__ void __launch_bounds__(256, MinBlocks3<Real, S, MODE, SRC>::value)
     if (x < p.nx && y < p.ny) sweep3_node<Real, S, SH, MODE, SRC>(p, x, y, blockIdx.z);
 }
 
+// ---------------------------------------------------------------- two nodes per thread, 16-bit storage
+// The scalar sweep of 16-bit storage is bound by instruction issue: 19 16-bit loads,
+// 18 of phi, 20 stores and their addresses per node.  Here a thread owns the nodes
+// x0, x0 + 1 (x0 even) of one row: per plane one 32-bit load brings the pair of the
+// source row (rows are padded to 64 elements, so it is aligned) and, for the ten
+// directions with c_x != 0, one 16-bit load the value beyond the pair; nine rows of
+// phi arrive as pairs, five of them with two values more; the results leave as 32-bit
+// stores (256^3 hill, FP16 local shift, 20 steps: 6.56 -> 5.36 ms, 63 GLUPS, 0.79 of
+// HBM).  The nodes' arithmetic and its order are the scalar sweep's, so the results
+// are equal bitwise.  Pairs that touch a bounce-back wall, or the half pair
+// at the end of an odd row, take the scalar path.
+template <typename S> __device__ __forceinline__ float pair_get(unsigned int w, int k);
+template <> __device__ __forceinline__ float pair_get<__half>(unsigned int w, int k) {
+    return __half2float(__ushort_as_half((unsigned short)(k ? w >> 16 : w & 0xffffu)));
+}
+template <> __device__ __forceinline__ float pair_get<__nv_bfloat16>(unsigned int w, int k) {
+    return __uint_as_float(k ? w & 0xffff0000u : w << 16);
+}
+template <typename S> __device__ __forceinline__ unsigned int pair_put(float a, float b);
+template <> __device__ __forceinline__ unsigned int pair_put<__half>(float a, float b) {
+    const __half2 h = __floats2half2_rn(a, b);
+    unsigned int w;
+    memcpy(&w, &h, 4);
+    return w;
+}
+template <> __device__ __forceinline__ unsigned int pair_put<__nv_bfloat16>(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    unsigned int w;
+    memcpy(&w, &h, 4);
+    return w;
+}
+
+// Four blocks per SM (64 registers): 5.36 ms on that hill, three 5.55, five 6.37.
+#ifndef BTRT3_VEC_MINBLOCKS
+#define BTRT3_VEC_MINBLOCKS 4
+#endif
+template <typename S, int SH, int MODE, int SRC>
+__global__ void __launch_bounds__(256, BTRT3_VEC_MINBLOCKS) sweep3_vec_kernel(const __grid_constant__ Sweep3Params<float> p) {
+    const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
+    if (x0 >= p.nx || y >= p.ny) return;
+    if (x0 + 1 >= p.nx || touches_wall3(p, x0, y, z) || touches_wall3(p, x0 + 1, y, z)) {
+#pragma unroll 1
+        for (int v = 0; v < 2 && x0 + v < p.nx; ++v) sweep3_node<float, S, SH, MODE, SRC>(p, x0 + v, y, z);
+        return;
+    }
+    const S *__restrict__ fin = static_cast<const S *>(p.fin);
+    S *__restrict__ fout = static_cast<S *>(p.fout);
+    const int node = z * p.slab + y * p.pitch + x0;
+    Near3 nb = near3(p, x0, y, z);
+    nb.xp = x0 + 2 == p.nx ? 2 - p.nx : 2;   // beyond the pair
+    // distance of the source row of direction i (c_y, c_z)
+    auto row = [&](int i) {
+        return (cz3(i) == 1 ? nb.zm : cz3(i) == -1 ? nb.zp : 0) + (cy3(i) == 1 ? nb.ym : cy3(i) == -1 ? nb.yp : 0);
+    };
+    unsigned int raw[19];
+    S edge[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) {
+        const int at = node + row(i);
+        raw[i] = *reinterpret_cast<const unsigned int *>(plane3_at<true, float, S>(p, fin, i, at));
+        if (cx3(i) == 1) edge[i] = *plane3_at<true, float, S>(p, fin, i, at + nb.xm);
+        if (cx3(i) == -1) edge[i] = *plane3_at<true, float, S>(p, fin, i, at + nb.xp);
+    }
+    // phi of the node's row (directions 1, 2) and, for the local shift, of the source
+    // rows: [row][x0 - 1 .. x0 + 2], rows named by one direction that comes from them
+    constexpr int kRowDir[9] = {0, 3, 4, 5, 6, 15, 16, 17, 18};
+    float ph[9][4];
+#pragma unroll
+    for (int r = 0; r < (SH == kShiftLocal ? 9 : 1); ++r) {
+        const int at = node + row(kRowDir[r]);
+        const float2 m = *reinterpret_cast<const float2 *>(p.phi_in + BTRT_IX(p.flags, at, p.plane));
+        ph[r][1] = m.x;
+        ph[r][2] = m.y;
+        if (SH == kShiftLocal && r < 5) {
+            ph[r][0] = p.phi_in[BTRT_IX(p.flags, at + nb.xm, p.plane)];
+            ph[r][3] = p.phi_in[BTRT_IX(p.flags, at + nb.xp, p.plane)];
+        }
+    }
+    bool bad = false;
+    float out[19], phi_o[2];
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+        const float phi_prev = ph[0][1 + v];
+        float d[19];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) {
+            const int k = v - cx3(i);   // 0, 1: of the pair; -1, 2: the value beyond it
+            d[i] = k < 0 || k > 1 ? Storage<S>::load(edge[i]) : pair_get<S>(raw[i], k);
+        }
+        if constexpr (SH == kShiftLocal) {
+#pragma unroll
+            for (int i = 1; i < 19; ++i) {
+                constexpr int kRow[3][3] = {{8, 4, 7}, {2, 0, 1}, {6, 3, 5}};   // [1 + c_z][1 + c_y]
+                d[i] = fma(wgt3<float>(i), ph[kRow[1 + cz3(i)][1 + cy3(i)]][1 + v - cx3(i)] - phi_prev, d[i]);
+            }
+        }
+        float srcv = 0.f;
+        if constexpr (SRC == kSrcConst) srcv = 1.f;
+        if constexpr (SRC == kSrcField) srcv = p.srcF[BTRT_IX(p.flags, node + v, p.plane)];
+        const float rs = SH == kShiftLocal ? phi_prev : p.phi_ref;
+        float phid;
+        phi_o[v] = collide3<float, MODE, SRC, SH>(p, d, rs, phi_prev, srcv, false, phid);
+        bad |= not_finite(phi_o[v]);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) {
+            const float t = SH == kShiftLocal ? fma(-wgt3<float>(i), phid, d[i]) : d[i];
+            if (v == 0) out[i] = t;
+            else *reinterpret_cast<unsigned int *>(const_cast<S *>(plane3_at<true, float, S>(p, fout, i, node))) =
+                     pair_put<S>(out[i], t);
+        }
+    }
+    *reinterpret_cast<float2 *>(p.phi_out + BTRT_IX(p.flags, node, p.plane)) = make_float2(phi_o[0], phi_o[1]);
+    if (bad) atomicOr(p.flags, 1);
+}
+
 }  // namespace btrt
