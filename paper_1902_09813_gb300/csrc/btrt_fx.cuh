@@ -191,10 +191,13 @@ BTRT_HD fx fx_ninth(fx x) {
 // (k2 - k0)/18 on (3/2) sigma and (k2 - k0)/4 on delta and Pi_xy; om2 = (1 - k0)/2.
 struct FxFold {
     FxConst Qxx, Qxy, Qyy, Px, Py, gx, gy, d18, d4, om2;
+    FxConst ux, uy, k06;   // per-node coefficients: u^ and k0/6
     int ok;          // kFxOk* bits; a form whose bit is not set takes the FP64 collision
     int pad;
+    double trh, detA;      // half the trace and the determinant of A0^
 };
-enum { kFxOkGeneral = 1, kFxOkLinear = 2 };   // om2 fits; all of the constants fit
+// om2, u^ and k0/6 fit; the constant-coefficient form's fit; bgx = bgy; c3 != 0
+enum { kFxOkGeneral = 1, kFxOkLinear = 2, kFxSameB = 4, kFxC3 = 8 };
 
 // Populations after the collision from the node's integer moments: a = k0 phi +
 // source, z the term of C(phi) != phi, X, Y = V/6, ks = (k2 - k0) sigma / 12, and the

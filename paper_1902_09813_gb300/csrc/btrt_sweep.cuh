@@ -468,18 +468,30 @@ __device__ __forceinline__ Real collide_fold(const SweepParams<Real> &p, Real (&
 
 // ---------------------------------------------------------------- the FP64 collision on the integer pipes
 // The FP64 form of collide_fold for one node, out of line: the nodes whose values
-// the integer form does not take, and the initialising collision.
+// the integer form does not take.  OWN: the source factor is sv, not p.src_val (many
+// steps per launch); the ordinary sweep's call carries no such argument (with it
+// the 8192^2 sweep was 5 % slower).
 template <int MODE, int SRC>
-static __device__ __noinline__ double collide_f64_slow(const SweepParams<double> &p, double *t, double phi_prev,
-                                                       double srcv, int node, double src_val) {
+__device__ __forceinline__ double collide_f64_plain(const SweepParams<double> &p, double *t, double phi_prev, double srcv,
+                                                    int node, const double *sv) {
     double d[9], phid;
 #pragma unroll
     for (int i = 0; i < 9; ++i) d[i] = t[i];
-    const double phi = collide_fold<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, node, phid,
-                                                                     nullptr, &src_val);
+    const double phi =
+        collide_fold<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, node, phid, nullptr, sv);
 #pragma unroll
     for (int i = 0; i < 9; ++i) t[i] = d[i];
     return phi;
+}
+template <int MODE, int SRC>
+static __device__ __noinline__ double collide_f64_slow(const SweepParams<double> &p, double *t, double phi_prev,
+                                                       double srcv, int node) {
+    return collide_f64_plain<MODE, SRC>(p, t, phi_prev, srcv, node, nullptr);
+}
+template <int MODE, int SRC>
+static __device__ __noinline__ double collide_f64_slow_own(const SweepParams<double> &p, double *t, double phi_prev,
+                                                           double srcv, int node, double sv) {
+    return collide_f64_plain<MODE, SRC>(p, t, phi_prev, srcv, node, &sv);
 }
 
 // 1/v by Householder's third-order iteration on the hardware's approximate
@@ -493,9 +505,9 @@ __device__ __forceinline__ double recip_f64(double v) {
 }
 
 // The per-node coefficient collision (kGeneral), or a reaction source: the moments
-// and the populations are integers as in fx_collide_linear, the nonlinear
-// coefficients and V are FP64 (44 operations instead of 97 with the two divisions
-// sharing one reciprocal).  Returns false, with d untouched, when a value leaves
+// and the populations are integers as in fx_collide_linear, and so is V given K1;
+// the nonlinear terms and K1 are FP64 (26 operations instead of 97; the two divisions
+// share one reciprocal).  Returns false, with d untouched, when a value leaves
 // the integer form's range.
 template <int MODE, int SRC>
 __device__ __forceinline__ bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], double phi_prev,
@@ -511,64 +523,88 @@ __device__ __forceinline__ bool fx_collide_general(const SweepParams<double> &p,
     fx X, Y, z = 0;
     FxConst d4, d18;
     if constexpr (MODE == kGeneral) {
-        const double jx = fx_to(m.jx, em), jy = fx_to(m.jy, em);
-        const double dphi = phi - phi_prev;
-        const double p2 = phi * phi;
-        double Bx, By, dBx, dBy;
+        // V = K1 (B - dB/2 - j) + k0 j + dB with B = u phi + bg g(phi), g = phi^q: the linear
+        // parts and j stay integers; g's mean (over phi, phi^{n-1}) and difference are FP64
+        const fx pv = fx_from(phi_prev, em);
+        double gs, gd;
         if (p.bq2) {
-            Bx = fma(p.ux, phi, p.bgx * p2);
-            By = fma(p.uy, phi, p.bgy * p2);
-            const double sp = phi + phi_prev;
-            dBx = fma(p.bgx, sp, p.ux) * dphi;
-            dBy = fma(p.bgy, sp, p.uy) * dphi;
+            const double p2 = phi * phi;
+            gd = (phi + phi_prev) * (phi - phi_prev);
+            gs = fma(-0.5, gd, p2);
         } else {
             const double gq = pow_half(phi, p.bq, p.bq_n, p.bq_h);
-            const double dg = gq - pow_half(phi_prev, p.bq, p.bq_n, p.bq_h);
-            Bx = fma(p.ux, phi, p.bgx * gq);
-            By = fma(p.uy, phi, p.bgy * gq);
-            dBx = fma(p.ux, dphi, p.bgx * dg);
-            dBy = fma(p.uy, dphi, p.bgy * dg);
+            gd = gq - pow_half(phi_prev, p.bq, p.bq_n, p.bq_h);
+            gs = fma(-0.5, gd, gq);
         }
-        if (p.c3 != 0.0) {
+        const double gsx = p.bgx * gs, gdx = p.bgx * gd;
+        double gsy = gsx, gdy = gdx;
+        if (!(p.fx.ok & kFxSameB)) {   // the flux direction is not (1, 1)
+            gsy = p.bgy * gs;
+            gdy = p.bgy * gd;
+        }
+        const unsigned int far = em + (1u << 20);
+        if (fx_exp(gsx) > far || fx_exp(gsy) > far || fx_exp(gdx) > far || fx_exp(gdy) > far) return false;
+        const FxArg mean = fx_arg((m.phi + pv) >> 1), diff = fx_arg(m.phi - pv);
+        const fx Ex = fx_mul(mean, p.fx.ux) + fx_from(gsx, em) - m.jx, Ey = fx_mul(mean, p.fx.uy) + fx_from(gsy, em) - m.jy;
+        const fx Dx = fx_mul(diff, p.fx.ux) + fx_from(gdx, em), Dy = fx_mul(diff, p.fx.uy) + fx_from(gdy, em);
+        const double p2 = phi * phi;
+        if (p.fx.ok & kFxC3) {
             // C(phi) - phi: in sigma, and k0 (C - phi) / 18 in the isotropic terms
             const double Cm = p.c3 * p2 * phi;
-            if (fx_exp(Cm) > em + (1u << 20)) return false;
+            if (fx_exp(Cm) > far) return false;
             m.s32 -= fx_from(Cm, em);
             z = fx_from(p.k0 * cst<double>(1, 18) * Cm, em);
         }
+        // K1 = adj(s A0^ + I/2) / det, s = 3 (1 + a2 phi^2): det and the trace are polynomials of
+        // s; 1/(6 det (2 tr - 1)) gives K1/6 and k2 (Eq. 62: 8/3 (tr - 1)/(2 tr - 1), tr - 1 = s trA)
         const double s3 = fma(L.a2x3, p2, 3.0);
-        double a0xx = p.A0xx, a0xy = p.A0xy, a0yy = p.A0yy;
+        double a0xx = p.A0xx, a0xy = p.A0xy, a0yy = p.A0yy, trh = p.fx.trh, detA = p.fx.detA;
         if (p.Af) {
             a0xx = p.Af[BTRT_IX(p.flags, node, p.plane)];
             a0xy = p.Af[BTRT_IX(p.flags, p.plane + node, 3 * p.plane)];
             a0yy = p.Af[BTRT_IX(p.flags, 2 * p.plane + node, 3 * p.plane)];
+            trh = 0.5 * (a0xx + a0yy);
+            detA = fma(a0xx, a0yy, -(a0xy * a0xy));
         }
-        const double mxx = fma(s3, a0xx, 0.5), mxy = s3 * a0xy, myy = fma(s3, a0yy, 0.5);
-        const double tr = mxx + myy;
-        const double det = fma(mxx, myy, -(mxy * mxy));
-        double id, k2;
+        const double det = fma(s3, fma(s3, detA, trh), 0.25);
+        double id6, dk;
         if (p.k2_hbb) {
-            const double q2 = fma(2.0, tr, -1.0);
-            const double rc = recip_f64(det * q2);
-            id = rc * q2;
-            k2 = (fma(cst<double>(8, 3), tr, -cst<double>(8, 3)) * det) * rc;
+            const double t = s3 * trh, q2 = fma(4.0, t, 1.0);
+            const double rc = recip_f64(det * fma(24.0, t, 6.0));
+            id6 = rc * q2;
+            dk = fma(32.0, (t * det) * rc, -p.k0);
         } else {
-            id = recip_f64(det);
-            k2 = p.k2c;
+            id6 = recip_f64(6.0 * det);
+            dk = p.k2c - p.k0;
         }
-        const double dk = k2 - p.k0;
-        const double ex = fma(-0.5, dBx, Bx - jx), ey = fma(-0.5, dBy, By - jy);
-        const double Kxx = myy * id, Kxy = -mxy * id, Kyy = mxx * id;
-        const double Vx = fma(Kxx, ex, fma(Kxy, ey, fma(p.k0, jx, dBx)));
-        const double Vy = fma(Kxy, ex, fma(Kyy, ey, fma(p.k0, jy, dBy)));
-        // also false for infinities and NaN
-        if (fx_exp(dk) > (1023u << 20) || fx_exp(Vx) > em + (2u << 20) || fx_exp(Vy) > em + (2u << 20)) return false;
+        const double half = fx_double(fx_bits(id6) - (1ull << 52)), si = s3 * id6;   // id6/2 by its exponent
+        const double Kxx = fma(si, a0yy, half), Kxy = -(si * a0xy), Kyy = fma(si, a0xx, half);
+        // K1/6 below 1/2 and k2 - k0 below 2 (also false for infinities and NaN), and the
+        // driving term below 2^61 units, which keeps the sums below in range
+        if (fx_exp(Kxx) > (1021u << 20) || fx_exp(Kxy) > (1021u << 20) || fx_exp(Kyy) > (1021u << 20) ||
+            fx_exp(dk) > (1023u << 20))
+            return false;
+        if ((unsigned int)((int)(Ex >> 32) + (1 << 29)) >= (1u << 30) || (unsigned int)((int)(Ey >> 32) + (1 << 29)) >= (1u << 30))
+            return false;
+        auto konst = [](double v, unsigned int one) {          // one: the exponent of the unit 2^-64
+            const FxArg c = fx_arg(fx_from(v, one));
+            return FxConst{c.h, c.l};
+        };
+        const FxConst kxx = konst(Kxx, 1017u << 20), kxy = konst(Kxy, 1017u << 20), kyy = konst(Kyy, 1017u << 20);
         const FxConst sixth = {0x2aaaaaab, (int)0xaaaaaaab};   // 2^64 / 6
-        X = fx_mul(fx_arg(fx_from(Vx, em)), sixth);
-        Y = fx_mul(fx_arg(fx_from(Vy, em)), sixth);
-        const FxArg c = fx_arg(fx_from(dk, 1019u << 20));      // dk / 4 in units of 2^-64
-        d4.hi = c.h;
-        d4.lo = c.l;
+        const FxArg ex = fx_arg(Ex), ey = fx_arg(Ey);
+        FxSum sx = fx_sum(), sy = fx_sum(), tx = fx_sum(), ty = fx_sum();
+        fx_add(sx, ex, kxx);
+        fx_add(sx, ey, kxy);
+        fx_add(sy, ex, kxy);
+        fx_add(sy, ey, kyy);
+        fx_add(tx, fx_arg(m.jx), p.fx.k06);
+        fx_add(tx, fx_arg(Dx), sixth);
+        fx_add(ty, fx_arg(m.jy), p.fx.k06);
+        fx_add(ty, fx_arg(Dy), sixth);
+        X = fx_value(sx) + fx_value(tx);
+        Y = fx_value(sy) + fx_value(ty);
+        d4 = konst(dk, 1019u << 20);                           // (k2 - k0) / 4
         d18 = d4;
         m.s32 = 2 * fx_ninth(m.s32);                           // (k2 - k0)/18 = (2/9) (k2 - k0)/4
     } else {
@@ -646,10 +682,11 @@ __device__ __forceinline__ void init_f64(const SweepParams<double> &p, double (&
 // integer form does not serve (a value out of its range, constants that do not
 // fit).  FP64 alone: 0.985 of the FP64 pipe at 10.4 GLUPS on the 8192^2
 // manufactured solution, 5.55 on the nonlinear workload; with the integer form
-// 37 GLUPS (0.89 of HBM) and 10.8.
-template <int MODE, int SRC>
+// 37 GLUPS (0.89 of HBM) and 13.
+template <int MODE, int SRC, bool OWN = false>
 __device__ __forceinline__ double collide_f64(const SweepParams<double> &p, double (&d)[9], double phi_prev,
-                                              double srcv, int node, double src_val) {
+                                              double srcv, int node, double sv = 0.0) {
+    const double src_val = OWN ? sv : p.src_val;
     constexpr bool LATE = SRC == kSrcReaction || SRC == kSrcRuntime;   // the source may depend on phi
     if (p.first) {
         double src = SRC != kSrcNone ? src_val * srcv : 0.0;
@@ -671,7 +708,8 @@ __device__ __forceinline__ double collide_f64(const SweepParams<double> &p, doub
         double t[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) t[i] = d[i];
-        phi = collide_f64_slow<MODE, SRC>(p, t, phi_prev, srcv, node, src_val);
+        if constexpr (OWN) phi = collide_f64_slow_own<MODE, SRC>(p, t, phi_prev, srcv, node, sv);
+        else phi = collide_f64_slow<MODE, SRC>(p, t, phi_prev, srcv, node);
 #pragma unroll
         for (int i = 0; i < 9; ++i) d[i] = t[i];
     }
@@ -890,11 +928,11 @@ template <> struct RowsPerThread<double, double> {
 // FP64 sweeps run on the integer pipes and need warps to cover load latency: five
 // blocks (48 registers) for k0 = 1 with constant coefficients measured 37.5 ms on
 // the 8192^2 manufactured solution (20 steps and the set-up), six 38.8; other k0 and
-// a reaction source would spill there, four and three blocks do not.  Per-node
-// coefficients: three blocks (80 registers), 2.95 ms on the 1001 x 777 nonlinear
-// workload against 3.14 with two.
+// a reaction source would spill there, four blocks do not.  Per-node coefficients:
+// four blocks (64 registers) 2.36 ms on the 1001 x 777 nonlinear workload, 40 steps,
+// three 2.53, two 3.17.
 #ifndef BTRT_MINBLOCKS_F64_GEN
-#define BTRT_MINBLOCKS_F64_GEN 3
+#define BTRT_MINBLOCKS_F64_GEN 4
 #endif
 // Double-word constant-coefficient sweeps: five blocks (48 registers, 12 spilled
 // bytes) measured 36.9 GLUPS against 33.5 with the compiler's 64 registers; the
@@ -1093,7 +1131,7 @@ __device__ __forceinline__ double finish_node(const SweepParams<Real> &p, int x,
     const Real rs = SC == kShiftLocal ? phi_prev : p.phi_ref;
     Real phid, phi;
     if constexpr (std::is_same<Real, double>::value) {
-        phi = collide_f64<MODE, SRC>(p, f, phi_prev, src, node, p.src_val);
+        phi = collide_f64<MODE, SRC>(p, f, phi_prev, src, node);
         phid = phi;
     } else {
         phi = collide_fold<Real, MODE, SRC, SC>(p, f, rs, phi_prev, src, p.first != 0, node, phid, Lc);

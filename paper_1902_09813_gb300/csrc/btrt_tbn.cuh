@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kTbnMaxThreads)
                         const Real rs = SC == kShiftLocal ? phi_prev : p.phi_ref;
                         Real phid, phi;
                         if constexpr (std::is_same<Real, double>::value) {
-                            phi = collide_f64<MODE, SRC>(p, d, phi_prev, srcv, node, src_val);
+                            phi = collide_f64<MODE, SRC, true>(p, d, phi_prev, srcv, node, src_val);
                             phid = phi;
                         } else {
                             phi = collide_fold<Real, MODE, SRC, SC>(p, d, rs, phi_prev, srcv, false, node, phid, nullptr,
