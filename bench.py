@@ -156,6 +156,8 @@ def kernel_form(args) -> str:
         return args.sweep
     large = args.n * args.n >= 1 << 21
     if args.shift in ("local_sr", "moment_sr"):
+        large = large or (args.shift == "moment_sr" and args.storage == "bf16" and args.workload == "mms"
+                          and args.n * args.n >= 7 << 17)
         return "vec" if large else "plain"
     return "vec" if args.storage in ("f16", "bf16") and large else "tb2"
 

@@ -421,12 +421,20 @@ int btrt::sweep_mode(btrt_lattice L) {
 // form from kVecAutoNodes on, the plain one below.  btrt_step takes small lattices
 // many steps per launch before it asks for this form (takes_tbn).
 constexpr long long kVecAutoNodes = 1LL << 21;
+// The first-moment form with BF16 storage and constant coefficients turns over earlier:
+// us per step, vector / plain, 800^2 16.7 / 15.2, 900^2 17.4 / 17.5, 1024^2 19.4 / 21.3 (FP16
+// 25.5 / 25.6, nonlinear BF16 24.6 / 21.5).
+constexpr long long kVecMomentNodes = 7LL << 17;
 int btrt::effective_sweep_variant(btrt_lattice L) {
     if (L->g.compute != BTRT_F32 || has_phi_lo(L->g)) return BTRT_SWEEP_PLAIN;
     if (L->sweep_variant != BTRT_SWEEP_AUTO) return L->sweep_variant;
     const bool s16 = L->g.storage == BTRT_F16 || L->g.storage == BTRT_BF16;
     const bool large = (long long)L->g.nx * L->g.ny >= kVecAutoNodes;
-    if (stochastic_store(L->g)) return large ? BTRT_SWEEP_VEC : BTRT_SWEEP_PLAIN;
+    if (stochastic_store(L->g)) {
+        const bool moment = has_j(L->g) && L->g.storage == BTRT_BF16 && sweep_mode(L) != kGeneral &&
+                            (long long)L->g.nx * L->g.ny >= kVecMomentNodes;
+        return large || moment ? BTRT_SWEEP_VEC : BTRT_SWEEP_PLAIN;
+    }
     return s16 && large ? BTRT_SWEEP_VEC : BTRT_SWEEP_TB2;
 }
 

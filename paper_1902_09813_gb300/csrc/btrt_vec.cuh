@@ -121,6 +121,13 @@ __device__ __forceinline__ float seg_value(const typename Vec4<S>::W &w, float e
 #ifndef BTRT_VEC_MINBLOCKS_S32
 #define BTRT_VEC_MINBLOCKS_S32 2
 #endif
+// First-moment form: three (80 registers); us per step at 4096^2, BF16 / FP16, two, three,
+// four blocks: manufactured solution 198 / 269, 178 / 248, 178 / 234, nonlinear 232 / 294,
+// 219 / 286, 231 / 298.  With the first moments read node by node (16 scalar loads each)
+// and two blocks it took 209 / 267 and 233 / 312.
+#ifndef BTRT_VEC_MINBLOCKS_MOMENT
+#define BTRT_VEC_MINBLOCKS_MOMENT 3
+#endif
 template <typename S> struct VecMinBlocks { static constexpr int value = BTRT_VEC_MINBLOCKS_S16; };
 template <> struct VecMinBlocks<float> { static constexpr int value = BTRT_VEC_MINBLOCKS_S32; };
 
@@ -168,6 +175,24 @@ __device__ __forceinline__ bool vec_interior(const SweepParams<float> &p, int x0
     }
 
     constexpr bool MOMENT = PullShift<SH>::value == kShiftMomentSR;
+    // first-moment form: the writers' first moments j of rows y - 1, y, y + 1, as the
+    // populations: a vector and two edge values per row and component (jy of the own row
+    // enters no direction)
+    W jraw[3][2];
+    float jl[3][2], jr[3][2];
+    if constexpr (MOMENT) {
+        const S *__restrict__ jin = static_cast<const S *>(p.j_in);
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (r == 1 && c == 1) continue;
+                const int at = c * p.plane + node + (r - 1) * p.pitch;
+                jraw[r][c] = ldg<L2ONLY>(reinterpret_cast<const W *>(jin + BTRT_IX(p.flags, at, 2 * p.plane)));
+                jl[r][c] = Storage<S>::load(ldg<L2ONLY>(jin + BTRT_IX(p.flags, at - 1, 2 * p.plane)));
+                jr[r][c] = Storage<S>::load(ldg<L2ONLY>(jin + BTRT_IX(p.flags, at + kVec, 2 * p.plane)));
+            }
+    }
     bool bad = false;
     float outv[9][kVec];
     float phi_o[kVec];
@@ -188,13 +213,15 @@ __device__ __forceinline__ bool vec_interior(const SweepParams<float> &p, int x0
             for (int i = 1; i < 9; ++i) f[i] = fma(wgt<float>(i), ph[1 - ey_of(i)][v - ex_of(i) + 1] - phi_prev, f[i]);
         }
         if constexpr (MOMENT) {
-            // the writers' first-moment terms, as pull_node adds them (scalar loads: L1 hits)
-            const S *jin = static_cast<const S *>(p.j_in);
+            // the writers' first-moment terms, as pull_node adds them
+            auto jv = [&](int r, int c, int k) {
+                const float t = k < 0 ? jl[r][c] : seg_value<S>(jraw[r][c], jr[r][c], k);
+                return DevScaled<S, SH>::value ? t * (1.f / kSrScaleF16) : t;
+            };
 #pragma unroll
             for (int i = 1; i < 9; ++i) {
-                const int nb = node + v - ey_of(i) * p.pitch - ex_of(i);
-                const float jx = dev_load<float, S, SH>(ldg<L2ONLY>(jin + BTRT_IX(p.flags, nb, 2 * p.plane)));
-                const float jy = dev_load<float, S, SH>(ldg<L2ONLY>(jin + BTRT_IX(p.flags, p.plane + nb, 2 * p.plane)));
+                const int r = 1 - ey_of(i), k = v - ex_of(i);
+                const float jx = ex_of(i) != 0 ? jv(r, 0, k) : 0.f, jy = ey_of(i) != 0 ? jv(r, 1, k) : 0.f;
                 f[i] = fma(w3<float>(i), e_dot<float>(i, jx, jy), f[i]);
             }
         }
@@ -363,8 +390,7 @@ __device__ __forceinline__ bool vec_tile_edges(const SweepParams<float> &p, int 
 // x0 = 4 (32 bx + tx) .. x0 + 3 of row y = 8 by + ty.  Never the initialising
 // collision and never a residual step (the host runs those in the plain form).
 template <typename S, int SH, int MODE, int SRC>
-// The first-moment form (more live values) is compiled for two blocks per SM.
-__global__ void __launch_bounds__(256, SH == kShiftMomentSR ? 2 : VecMinBlocks<S>::value)
+__global__ void __launch_bounds__(256, SH == kShiftMomentSR ? BTRT_VEC_MINBLOCKS_MOMENT : VecMinBlocks<S>::value)
     sweep_vec_kernel(const __grid_constant__ SweepParams<float> p) {
     const int x0 = (blockIdx.x * blockDim.x + threadIdx.x) * kVec;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
