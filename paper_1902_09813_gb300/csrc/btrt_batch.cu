@@ -108,30 +108,32 @@ __device__ __forceinline__ bool grid_barrier(unsigned int *count, unsigned int t
     return ok != 0;
 }
 
-// Member m was frozen by an earlier btrt_batch_step_tol (word 1 of its lattice's
-// device flags): launches leave it as it is.  The mark changes only between
-// launches, so every thread of a block reads the same value.
+// Copy member M's parameters into shared memory and patch the step-dependent ones:
+// buffer parity (flips since the slice began) and the source and wall time factors of
+// step k of the slice from the host-computed step table.  Returns true when the
+// member was frozen by an earlier btrt_batch_step_tol (word 1 of its lattice's device
+// flags; the mark changes only between launches, so every thread reads the same
+// value): launches leave it as it is.  Everything the patch needs is loaded beside
+// the copy, and the frozen mark through the copied pointer while the patch runs: a
+// tile waits for two global loads one after the other (the copy, the mark), not four
+// (64 members, 100 steps: 11.15 -> 10.96 ms).  The function begins and ends with a barrier.
 template <typename Real>
-__device__ __forceinline__ bool member_frozen(const BatchArgs<Real> &a, int m) {
-    return (a.members[m].p.flags[1] & 1) != 0;
-}
-
-// One tile of one step: load the member's parameters into shared memory, patch
-// the step-dependent ones (buffer parity, source and wall time factors from the
-// host-computed step table) and sweep the tile's nodes.  LIN: every member of
-// the batch takes the constant-coefficient collision and a source other than
-// the reaction term, so only that collision and those sources are compiled
-// (fewer registers than the form that can take any member).
-// Copy member M's parameters into shared memory and patch the step-dependent
-// ones: buffer parity (flips since the slice began) and the source and wall time
-// factors of step k of the slice from the host-computed step table.  The caller
-// places no barrier before reading sp; this function ends with one.
-template <typename Real>
-__device__ __forceinline__ void stage_member(const BatchArgs<Real> &a, int member, int k, int flip,
+__device__ __forceinline__ bool stage_member(const BatchArgs<Real> &a, int member, int k, int flip,
                                              SweepParams<Real> &sp) {
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int nthr = blockDim.x * blockDim.y;
     const BatchMember<Real> &M = a.members[member];
+    int cur = 0;
+    long long step = 0;
+    Real src_val = Real(0), wall_fac = Real(0);
+    if (tid == 0) {
+        cur = (M.cur + flip) & 1;            // buffer flips since the slice began
+    } else if (tid == 32) {
+        const Real *v = a.step_vals + ((size_t)member * a.table_steps + k) * 2;
+        src_val = v[0];
+        wall_fac = v[1];
+        step = M.step;
+    }
     __syncthreads();   // the previous tile is done with sp
     {
         const int *src = reinterpret_cast<const int *>(&M.p);
@@ -139,24 +141,24 @@ __device__ __forceinline__ void stage_member(const BatchArgs<Real> &a, int membe
         for (int w = tid; w < (int)(sizeof(SweepParams<Real>) / 4); w += nthr) dst[w] = src[w];
     }
     __syncthreads();
+    const bool frozen = (sp.flags[1] & 1) != 0;
     if (tid == 0) {
-        const int cur = (M.cur + flip) & 1;  // buffer flips since the slice began
-        const void *b0 = M.p.fin;            // buffer 0
-        void *b1 = M.p.fout;                 // buffer 1
-        sp.fin = cur ? b1 : b0;
-        sp.fout = cur ? const_cast<void *>(b0) : b1;
-        const Real *q0 = M.p.phi_in;         // phi plane 0
-        Real *q1 = M.p.phi_out;              // phi plane 1
-        sp.phi_in = cur ? q1 : q0;
-        sp.phi_out = cur ? const_cast<Real *>(q0) : q1;
+        if (cur) {                           // buffer 1 holds the current populations and phi
+            const void *b0 = sp.fin;
+            sp.fin = sp.fout;
+            sp.fout = const_cast<void *>(b0);
+            const Real *q0 = sp.phi_in;
+            sp.phi_in = sp.phi_out;
+            sp.phi_out = const_cast<Real *>(q0);
+        }
     } else if (tid == 32) {
-        const Real *v = a.step_vals + ((size_t)member * a.table_steps + k) * 2;
-        sp.src_val = v[0];
-        sp.wall_fac = v[1];
+        sp.src_val = src_val;
+        sp.wall_fac = wall_fac;
         sp.first = 0;
-        sp.sr_seed = sr_step_seed(M.step + k + 1);   // stochastic rounding: the seed of this step
+        sp.sr_seed = sr_step_seed(step + k + 1);   // stochastic rounding: the seed of this step
     }
     __syncthreads();
+    return frozen;
 }
 
 // One tile of one step: stage the member's parameters (stage_member) and sweep
@@ -169,15 +171,14 @@ __device__ __forceinline__ void batch_tile(const BatchArgs<Real> &a, int t, int 
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int nthr = blockDim.x * blockDim.y;
     const int4 tile = a.tiles[t];
-    if (member_frozen(a, tile.x)) return;
-    const BatchMember<Real> &M = a.members[tile.x];
-    stage_member(a, tile.x, k, flip, sp);
+    const int mode = LIN ? kLinear : a.members[tile.x].mode;
+    if (stage_member(a, tile.x, k, flip, sp)) return;
     const SweepParams<Real> &lp = sp;
     const int x = tile.y + threadIdx.x;
     double r = 0.0;
     if (x < lp.nx) {
         const int y0 = tile.z + threadIdx.y;
-        if (!LIN && M.mode == kGeneral) {
+        if (!LIN && mode == kGeneral) {
             if (resid) r = sweep_rows<Real, S, SH, kGeneral, kSrcRuntime, L2ONLY, true>(lp, x, y0, blockDim.y, a.rows);
             else sweep_rows<Real, S, SH, kGeneral, kSrcRuntime, L2ONLY, false>(lp, x, y0, blockDim.y, a.rows);
         } else {
@@ -258,10 +259,9 @@ __global__ void __launch_bounds__(256, LIN ? BatchVecMinBlocks<S>::value : 2)
     __shared__ SweepParams<float> sp;
     const BatchArgs<float> &a = va.a;
     const int4 tile = a.tilesv[va.t0 + blockIdx.x];
-    if (member_frozen(a, tile.x)) return;
-    const int mode = a.members[tile.x].mode;
+    const int mode = LIN ? kLinear : a.members[tile.x].mode;
     const FoldConsts<float> *Lc = &va.lin[tile.x - va.m0];
-    stage_member(a, tile.x, k, flip, sp);
+    if (stage_member(a, tile.x, k, flip, sp)) return;
     const SweepParams<float> &lp = sp;
     const int x0 = tile.y + threadIdx.x * kVec;
     bool bad = false;
@@ -307,8 +307,8 @@ __global__ void __launch_bounds__(256, LIN ? BTRT_BATCH_TB2_MINBLOCKS_LIN : BTRT
     extern __shared__ float tb_smem[];
     const int tid = threadIdx.x;
     const int4 tile = a.tiles2[blockIdx.x];
-    if (member_frozen(a, tile.x)) return;
     const BatchMember<float> &M = a.members[tile.x];
+    if (M.p.flags[1] & 1) return;   // frozen (stage_member)
     {
         const int *src = reinterpret_cast<const int *>(&M.p);
         int *da = reinterpret_cast<int *>(&spa), *db = reinterpret_cast<int *>(&spb);
