@@ -88,8 +88,9 @@ __device__ __forceinline__ bool tbn_barrier(unsigned int *count, unsigned int ta
     __syncthreads();
     int good = 1;
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(count, 1u);
+        // releases the block's writes (ordered before by the barrier above); the acquiring
+        // load and the barrier below order every thread's later loads
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
         unsigned long long polls = 0;
         unsigned int seen;
         do {
@@ -100,7 +101,6 @@ __device__ __forceinline__ bool tbn_barrier(unsigned int *count, unsigned int ta
                 break;
             }
         } while (seen < target);
-        __threadfence();
     }
     return __syncthreads_and(good) != 0;
 }

@@ -78,3 +78,12 @@ def test_residual_and_non_finite_flag():
     a.init(phi0).step(6)
     with pytest.raises(C.BtrtError):
         a.check()
+
+
+@pytest.mark.parametrize("size", [(49, 33), (50, 41), (32, 400), (700, 33), (97, 57)], ids=str)
+@pytest.mark.parametrize("form", FORMS[:1] + FORMS[2:3] + FORMS[-1:], ids=lambda f: "-".join(f))
+def test_narrow_last_tiles(size, form):
+    """Last tiles of one to a few nodes: a region then reaches over them into the next
+    tile, on periodic axes round the lattice."""
+    p = w.random_state_problem(*size, seed=8, nonlinear=False, source="none")
+    _same(p, form, (41,))
