@@ -153,8 +153,19 @@ __device__ __forceinline__ void tbn_pull(const SweepParams<Real> &p, Real wall_f
 
 // st.n steps: p holds the parameters of the first (its inputs in fin, phi_in; the
 // other buffers in fout, phi_out; the rounds swap them).
+// Threads and resident blocks per SM the kernel is compiled for.  FP32 compute: two
+// blocks of 512 (64 registers), so that four of 256 fit as well: us per step at 256^2,
+// FP32 storage, manufactured solution / nonlinear 2.45 / 2.35 against 4.03 / 3.97 with the
+// compiler's 80 registers (64^2: 1.59 / 1.45 against 1.54 / 1.42).  Double-word, constant
+// coefficients: three of 256, 181^2 3.1 against 4.3 with two; its per-node coefficients
+// (160^2 3.5 against 4.6 with three) and FP64 (64^2 hill 2.0 against 2.1) two.
+template <typename Real, int MODE> struct TbnBounds {
+    static constexpr int threads = sizeof(Real) == 4 ? kTbnMaxThreads : 256;
+    static constexpr int blocks = std::is_same<Real, dw>::value && MODE != kGeneral ? 3 : 2;
+};
+
 template <typename Real, typename S, int SH, int MODE, int SRC>
-__global__ void __launch_bounds__(kTbnMaxThreads)
+__global__ void __launch_bounds__(TbnBounds<Real, MODE>::threads, TbnBounds<Real, MODE>::blocks)
     sweep_tbn_kernel(const __grid_constant__ SweepParams<Real> p, const __grid_constant__ TbnSteps<Real> st) {
     using G = TbnGeom<Real, SH>;
     constexpr int SC = CollShift<SH>::value, PL = G::PLANE;
