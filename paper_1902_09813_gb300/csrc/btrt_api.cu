@@ -472,7 +472,8 @@ btrt_status launch(btrt_lattice L, int64_t n, bool first, bool resid = false) {
 // launch against the form AUTO takes otherwise (square lattices, 200 steps with set-up
 // and read): FP32 storage 64^2 1.7 / 5.2, 256^2 2.6 / 5.2, 362^2 3.8 / 5.3, 430^2 5.7 / 5.3;
 // FP16 local shift 64^2 1.8 / 6.3, 362^2 3.9 / 6.3, 512^2 6.5 / 7.3 (nonlinear 6.8 / 9.4);
-// double-word phi 512^2 7.1 / 10.4, first-moment form 8.3 / 10.4; FP64 hill 64^2 2.1 / 6.3,
+// double-word phi 512^2 6.6 / 10.4, with constant coefficients 540^2 8.4 / 10.4, 640^2
+// 10.9 / 12.5, 724^2 10.9 / 13.2; first-moment form 512^2 7.8 / 10.4; FP64 hill 64^2 2.1 / 6.3,
 // 160^2 3.1 / 6.3, 181^2 5.0 / 6.3, 256^2 6.9 / 6.3, nonlinear 160^2 10.2 / 12.3, 181^2
 // 14.8 / 12.4; double-word format hill 256^2 6.1 / 6.3, nonlinear 181^2 6.2 / 6.3.
 bool takes_tbn(btrt_lattice L) {
@@ -483,7 +484,7 @@ bool takes_tbn(btrt_lattice L) {
     if (g.compute == BTRT_F64) most = general ? 3 << 13 : 1 << 15;
     else if (g.compute == BTRT_DF64) most = general ? 1 << 15 : 1 << 16;
     else if (g.storage == BTRT_F32 && !has_phi_lo(g)) most = 1 << 17;
-    else most = 1 << 18;
+    else most = g.storage == BTRT_F32 && !general ? 1 << 19 : 1 << 18;
     return (long long)g.nx * g.ny <= most;
 }
 

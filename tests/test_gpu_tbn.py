@@ -87,3 +87,9 @@ def test_narrow_last_tiles(size, form):
     tile, on periodic axes round the lattice."""
     p = w.random_state_problem(*size, seed=8, nonlinear=False, source="none")
     _same(p, form, (41,))
+
+
+@pytest.mark.parametrize("size", [(723, 725), (513, 512), (130, 4001)], ids=str)
+def test_largest_double_word_phi(size):
+    p = w.random_state_problem(*size, seed=9, bc=(1, 1, 0, 0), nonlinear=False, source="trig")
+    _same(p, ("f32", "f32", "local_dw"), (9,))
