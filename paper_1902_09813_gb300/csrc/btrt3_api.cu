@@ -238,31 +238,10 @@ void fill3(btrt3_lattice L, Sweep3Params<Real> &p, int64_t n, bool first) {
         p.k0_one = k0 == 1.0 ? 1 : 0;
     }
     if constexpr (std::is_same<Real, double>::value) {
-        // the same constants for the integer collision (as in two dimensions)
-        const double dk = L->k2 - c.k0;
-        const double v[16] = {-p.Q[0],           -p.K1[1],           -p.K1[2],           -p.Q[1], -p.K1[4], -p.Q[2],
-                              p.Ku[0] + p.gu[0], p.Ku[1] + p.gu[1], p.Ku[2] + p.gu[2], -p.gu[0], -p.gu[1], -p.gu[2],
-                              dk,                dk,                dk,                p.om};
-        const int div[16] = {6, 6, 6, 6, 6, 6, 6, 6, 6, 6, 6, 6, 12, 24, 4, 2};
-        FxConst k[16];
-        bool ok = true;
-        for (int i = 0; i < 16; ++i) {
-            const bool fits = std::fabs(v[i]) < 0.4999 * div[i];
-            k[i] = fx_const(fits ? v[i] : 0.0, div[i]);
-            ok = ok && fits;
-        }
-        ok = ok && fx_flux_fits3(k[0], k[1], k[2], k[6], k[9]) && fx_flux_fits3(k[1], k[3], k[4], k[7], k[10]) &&
-             fx_flux_fits3(k[2], k[4], k[5], k[8], k[11]);
-        for (int i = 0; i < 6; ++i) p.fx.Q[i] = k[i];
-        for (int i = 0; i < 3; ++i) {
-            p.fx.P[i] = k[6 + i];
-            p.fx.g[i] = k[9 + i];
-        }
-        p.fx.d12 = k[12];
-        p.fx.d24 = k[13];
-        p.fx.d4 = k[14];
-        p.fx.om2 = k[15];
-        p.fx.ok = (std::fabs(p.om) < 0.9998 ? kFxOkGeneral : 0) | (ok ? kFxOkLinear : 0);
+        // the same constants for the integer collision
+        p.fx = fx_fold3({p.Q[0], p.K1[1], p.K1[2], p.Q[1], p.K1[4], p.Q[2]},
+                        {p.Ku[0] + p.gu[0], p.Ku[1] + p.gu[1], p.Ku[2] + p.gu[2]}, {p.gu[0], p.gu[1], p.gu[2]},
+                        L->k2 - c.k0, p.om);
     }
     p.cond_limit = (Real)1.0e6;
     for (int k = 0; k < 6; ++k) p.A0d[k] = L->A0[k];

@@ -369,24 +369,12 @@ void btrt::fill_params(btrt_lattice L, SweepParams<Real> &p, int64_t n, bool fir
         q.a2x3 = (Real)(3.0 * c.a2);
     }
     if constexpr (std::is_same<Real, double>::value) {
-        // the same constants for the integer collision; where one does not fit (or is
-        // not finite), the kernels keep the FP64 form
+        // the same constants for the integer collision
         const FoldConsts<double> &q = p.lin;
-        const double dk = L->k2 - c.k0;
-        const double v[13] = {-q.Qxx, -q.Qxy, -q.Qyy, q.Pgx, q.Pgy, -q.gx, -q.gy, dk, dk, q.om, L->ux, L->uy, c.k0};
-        const int div[13] = {6, 6, 6, 6, 6, 6, 6, 18, 4, 2, 1, 1, 6};
-        FxConst k[13];
-        bool fit[13];
-        for (int i = 0; i < 13; ++i) {
-            fit[i] = std::fabs(v[i]) < 0.4999 * div[i];
-            k[i] = fx_const(fit[i] ? v[i] : 0.0, div[i]);
-        }
-        bool lin = fx_flux_fits(k[0], k[1], k[3], k[5]) && fx_flux_fits(k[1], k[2], k[4], k[6]);
-        for (int i = 0; i < 10; ++i) lin = lin && fit[i];
-        const int ok = (fit[9] && fit[10] && fit[11] && fit[12] ? kFxOkGeneral : 0) | (lin ? kFxOkLinear : 0) |
-                       (L->bgx == L->bgy ? kFxSameB : 0) | (c.c3 != 0.0 ? kFxC3 : 0);
-        p.fx = FxFold{k[0], k[1], k[2], k[3],  k[4],  k[5],  k[6], k[7],
-                      k[8], k[9], k[10], k[11], k[12], ok, 0, 0.5 * (L->A0[0] + L->A0[2]), L->A0[0] * L->A0[2] - L->A0[1] * L->A0[1]};
+        p.fx = fx_fold({q.Qxx, q.Qxy, q.Qyy}, {q.Pgx, q.Pgy}, {q.gx, q.gy}, L->k2 - c.k0, q.om, {L->ux, L->uy}, c.k0);
+        p.fx.ok |= (L->bgx == L->bgy ? kFxSameB : 0) | (c.c3 != 0.0 ? kFxC3 : 0);
+        p.fx.trh = 0.5 * (L->A0[0] + L->A0[2]);
+        p.fx.detA = L->A0[0] * L->A0[2] - L->A0[1] * L->A0[1];
     }
     // the reference value of kShiftRef storage (zero otherwise)
     p.phi_ref = shift_of(g) == kShiftRef ? (Real)g.phi_ref : (Real)0.0;

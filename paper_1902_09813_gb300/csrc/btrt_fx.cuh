@@ -199,6 +199,86 @@ struct FxFold {
 // om2, u^ and k0/6 fit; the constant-coefficient form's fit; bgx = bgy; c3 != 0
 enum { kFxOkGeneral = 1, kFxOkLinear = 2, kFxSameB = 4, kFxC3 = 8 };
 
+// A constant as the products see it.
+inline double fx_real(const FxConst &c) { return ldexp((double)c.hi, -32) + ldexp((double)c.lo, -64); }
+
+// Whether every sum of fx_collide_linear stays in its word, beyond what fx_density and
+// fx_flux_fits cover: the fluxes V/6 and the results, as linear maps of the populations
+// (at most 1, in units of 2^59), phi^{n-1} (4) and the source (2), the word ending at 16.
+inline bool fx_linear_fits(const FxFold &q) {
+    const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+    const double Qxx = fx_real(q.Qxx), Qxy = fx_real(q.Qxy), Qyy = fx_real(q.Qyy);
+    const double Px = fx_real(q.Px), Py = fx_real(q.Py), gx = fx_real(q.gx), gy = fx_real(q.gy);
+    const double d18 = fx_real(q.d18), d4 = fx_real(q.d4), om = 2.0 * fx_real(q.om2);
+    double top = 6.0 * (fabs(Qxx) + fabs(Qxy)) + 9.0 * fabs(Px) + 4.0 * fabs(gx);
+    top = fmax(top, 6.0 * (fabs(Qyy) + fabs(Qxy)) + 9.0 * fabs(Py) + 4.0 * fabs(gy)) + 0.5;   // X, Y: 2 max(|X|, |Y|) < 16
+    bool fits = top < 8.0;
+    for (int i = 0; i < 9; ++i) {
+        const double w = i == 0 ? 4.0 / 9 : (i <= 4 ? 1.0 / 9 : 1.0 / 36);
+        const int axis = i >= 1 && i <= 4, diag = i > 4;
+        double sum = 2.0 * w + 4.0 * 18.0 * w * fabs(ex[i] * gx + ey[i] * gy) + 0.01;
+        for (int k = 0; k < 9; ++k) {
+            const double jx = ex[k], jy = ey[k], pxy = ex[k] * ey[k], del = ex[k] * ex[k] - ey[k] * ey[k];
+            const double s32 = k == 0 ? -1.0 : (k <= 4 ? 0.5 : 2.0), ks = d18 * s32;
+            const double X = Qxx * jx + Qxy * jy + Px, Y = Qxy * jx + Qyy * jy + Py;
+            double r = (k == i ? om : 0.0) + w * (1.0 - om) + 18.0 * w * (ex[i] * X + ey[i] * Y);
+            r += i == 0 ? 8.0 * ks : -ks;
+            if (axis) r -= (ex[i] * ex[i] - ey[i] * ey[i]) * d4 * del;
+            if (diag) r -= ex[i] * ey[i] * d4 * pxy;
+            sum += fabs(r);
+        }
+        fits = fits && sum < 16.0;
+    }
+    return fits;
+}
+
+// The fold of a lattice: Q = K1 - k0 I (xx, xy, yy), P = K1 u^ + g, g, k2 - k0, 1 - k0, u^
+// and k0.  A constant that does not fit (or is not finite), or a sum that could leave its
+// word, clears the form's bit: the kernels then keep the FP64 collision.
+// Per-node coefficients need no such test (units of 2^59, |u^| < 1): over k0 and k2 in
+// (0, 2) the populations' part of a result, with k0 j/6 of the flux, and the source take
+// at most 9.9 (rest direction), 4 (axes) and 1.8; C - phi, tested against 2, takes 1.8, 0.5
+// and 0.5; the rest of the flux, (K1 E + B's change)/6, enters the axes with 2 (9.7 + 13 |u^| + 2)/6
+// = 8.3, since K1's eigenvalues lie in (0, 2) and E is tested against 4.
+inline FxFold fx_fold(const double (&Q)[3], const double (&P)[2], const double (&g)[2], double dk, double om,
+                      const double (&u)[2], double k0) {
+    const double v[13] = {-Q[0], -Q[1], -Q[2], P[0], P[1], -g[0], -g[1], dk, dk, om, u[0], u[1], k0};
+    const int div[13] = {6, 6, 6, 6, 6, 6, 6, 18, 4, 2, 1, 1, 6};
+    FxConst k[13];
+    bool fit[13], lin = true;
+    for (int i = 0; i < 13; ++i) {
+        fit[i] = fabs(v[i]) < 0.4999 * div[i];
+        k[i] = fx_const(fit[i] ? v[i] : 0.0, div[i]);
+        if (i < 10) lin = lin && fit[i];
+    }
+    FxFold q = {k[0], k[1], k[2], k[3], k[4], k[5], k[6], k[7], k[8], k[9], k[10], k[11], k[12], 0, 0, 0.0, 0.0};
+    lin = lin && fx_flux_fits(q.Qxx, q.Qxy, q.Px, q.gx) && fx_flux_fits(q.Qxy, q.Qyy, q.Py, q.gy) && fx_linear_fits(q);
+    q.ok = (fit[9] && fit[10] && fit[11] && fit[12] ? kFxOkGeneral : 0) | (lin ? kFxOkLinear : 0);
+    return q;
+}
+
+// Sums whose terms may pass 2^63 (the caller tests the result before it is used).
+BTRT_HD fx fx_plus(fx a, fx b) { return (fx)((unsigned long long)a + (unsigned long long)b); }
+BTRT_HD fx fx_minus(fx a, fx b) { return (fx)((unsigned long long)a - (unsigned long long)b); }
+
+// a = k0 phi + source of a node; false when it could leave its word.  With k0 = 1 it
+// cannot (nine populations below 2^59 units and a source below 2^60; in three dimensions
+// nineteen below 2^58, and 2^59).  Otherwise half of it is formed again from the high
+// words of its terms, which fits: three cut words, three units of 2^32 off.
+template <bool K0ONE, bool SOURCE, int TOP>
+BTRT_HD bool fx_density(fx phi, const FxArg &ph, const FxConst &om2, double src, unsigned int em, fx &a) {
+    const fx s = SOURCE ? fx_from<TOP>(src, em) : 0;
+    if (K0ONE) {
+        a = phi + s;
+        return true;
+    }
+    const fx om = fx_mul(ph, om2);
+    a = fx_plus(fx_minus(phi, 2 * om), s);
+    const int half = ((int)(phi >> 32) >> 1) - (int)(om >> 32) + ((int)(s >> 32) >> 1);
+    constexpr unsigned int most = (1u << 30) - 4u;
+    return (unsigned int)half + most < 2u * most;
+}
+
 // Populations after the collision from the node's integer moments: a = k0 phi +
 // source, z the term of C(phi) != phi, X, Y = V/6, ks = (k2 - k0) sigma / 12, and the
 // two anisotropic second-order terms t1 = (k2 - k0) delta / 4, t5 = (k2 - k0) Pi_xy / 4.
@@ -206,7 +286,7 @@ BTRT_HD void fx_expand(fx a, fx z, fx X, fx Y, fx ks, fx t1, fx t5, fx (&r)[9]) 
     const fx b = fx_ninth(a);
     const fx zk = z - ks;
     const fx T1 = b + zk, T5 = (b >> 2) + zk;
-    r[0] = a - 4 * (T1 + T5);           // the other eight sum to 4 (T1 + T5)
+    r[0] = fx_minus(a, 4 * (T1 + T5));  // the other eight sum to 4 (T1 + T5)
     const fx A1 = T1 - t1, A2 = T1 + t1;
     r[1] = A1 + 2 * X;
     r[3] = A1 - 2 * X;
@@ -294,10 +374,8 @@ BTRT_HD bool fx_collide_linear(const FxFold &q, double (&d)[9], double phi_prev,
     fx_add(sy, ph, q.Py);
     fx_add(sy, pp, q.gy);
     const fx ks = fx_mul(fx_arg(m.s32), q.d18), t1 = fx_mul(fx_arg(m.del), q.d4), t5 = fx_mul(fx_arg(m.pxy), q.d4);
-    fx a = m.phi;
-    if (!K0ONE) a -= 2 * fx_mul(ph, q.om2);
-    if (SOURCE) a += fx_from(src, em);
-    fx r[9];
+    fx a, r[9];
+    if (!fx_density<K0ONE, SOURCE, 58>(m.phi, ph, q.om2, src, em, a)) return false;
     fx_expand(a, 0, fx_value(sx), fx_value(sy), ks, t1, t5, r);
     fx_store<K0ONE, BTRT_FX_NADD>(D, r, q.om2, em, d);
     phi_out = fx_to(m.phi, em);
@@ -333,6 +411,78 @@ inline bool fx_flux_fits3(const FxConst &qx, const FxConst &qy, const FxConst &q
     return t < 9223372036854775808.0;
 }
 
+// As fx_linear_fits: populations at most 1 (in units of 2^58), phi^{n-1} 4, the source 2,
+// the word ending at 32.
+inline bool fx_linear_fits3(const FxFold3 &q) {
+    const int c[19][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0}, {0, 0, 1},  {0, 0, -1},
+                          {1, 1, 0},  {-1, 1, 0}, {1, -1, 0}, {-1, -1, 0}, {1, 0, 1},  {-1, 0, 1}, {1, 0, -1},
+                          {-1, 0, -1}, {0, 1, 1}, {0, -1, 1}, {0, 1, -1},  {0, -1, -1}};
+    const int at[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+    double Q[3][3], P[3], g[3], top = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        P[a] = fx_real(q.P[a]);
+        g[a] = fx_real(q.g[a]);
+        double t = 19.0 * fabs(P[a]) + 4.0 * fabs(g[a]) + 0.5;
+        for (int b = 0; b < 3; ++b) {
+            Q[a][b] = fx_real(q.Q[at[a][b]]);
+            t += 10.0 * fabs(Q[a][b]);
+        }
+        top = fmax(top, t);
+    }
+    bool fits = top < 16.0;   // X, Y, Z: twice the largest < 32
+    const double d4 = fx_real(q.d4), om = 2.0 * fx_real(q.om2);
+    for (int i = 0; i < 19; ++i) {
+        const double w = i == 0 ? 1.0 / 3 : (i <= 6 ? 1.0 / 18 : 1.0 / 36);
+        double cg = 0.0;
+        for (int a = 0; a < 3; ++a) cg += c[i][a] * g[a];
+        double sum = 2.0 * w + 4.0 * 18.0 * w * fabs(cg) + 0.01;
+        for (int k = 0; k < 19; ++k) {
+            // w (a + 3 c.V - (9/2) (k2 - k0) (c c : N - t3)), N = sum c c d - phi I / 3, t3 = tr N / 3
+            double V = 0.0, H = 0.0, e2 = 0.0, t3 = 0.0;
+            for (int a = 0; a < 3; ++a) {
+                double X = P[a];
+                for (int b = 0; b < 3; ++b) {
+                    X += Q[a][b] * c[k][b];
+                    H += c[i][a] * c[i][b] * (c[k][a] * c[k][b] - (a == b ? 1.0 / 3 : 0.0));
+                }
+                V += c[i][a] * X;
+                e2 += c[k][a] * c[k][a];
+            }
+            t3 = (e2 - 1.0) / 3.0;
+            sum += fabs((k == i ? om : 0.0) + w * (1.0 - om) + 18.0 * w * V - 18.0 * w * d4 * (H - t3));
+        }
+        fits = fits && sum < 32.0;
+    }
+    return fits;
+}
+
+// As fx_fold: Q = K1 - k0 I (xx, xy, xz, yy, yz, zz), P = K1 u^ + g, g, k2 - k0, 1 - k0.
+inline FxFold3 fx_fold3(const double (&Q)[6], const double (&P)[3], const double (&g)[3], double dk, double om) {
+    const double v[16] = {-Q[0], -Q[1], -Q[2], -Q[3], -Q[4], -Q[5], P[0], P[1], P[2], -g[0], -g[1], -g[2], dk, dk, dk, om};
+    const int div[16] = {6, 6, 6, 6, 6, 6, 6, 6, 6, 6, 6, 6, 12, 24, 4, 2};
+    FxConst k[16];
+    bool ok = true;
+    for (int i = 0; i < 16; ++i) {
+        const bool fits = fabs(v[i]) < 0.4999 * div[i];
+        k[i] = fx_const(fits ? v[i] : 0.0, div[i]);
+        ok = ok && fits;
+    }
+    FxFold3 q = {};
+    for (int i = 0; i < 6; ++i) q.Q[i] = k[i];
+    for (int i = 0; i < 3; ++i) {
+        q.P[i] = k[6 + i];
+        q.g[i] = k[9 + i];
+    }
+    q.d12 = k[12];
+    q.d24 = k[13];
+    q.d4 = k[14];
+    q.om2 = k[15];
+    ok = ok && fx_flux_fits3(k[0], k[1], k[2], k[6], k[9]) && fx_flux_fits3(k[1], k[3], k[4], k[7], k[10]) &&
+         fx_flux_fits3(k[2], k[4], k[5], k[8], k[11]) && fx_linear_fits3(q);
+    q.ok = (fabs(om) < 0.9998 ? kFxOkGeneral : 0) | (ok ? kFxOkLinear : 0);
+    return q;
+}
+
 struct FxMoments3 {
     fx phi, jx, jy, jz, pxy, pxz, pyz;
     fx hx, hy, t3;   // 3 h_x, 3 h_y (h_z = -h_x - h_y) and 3 t3
@@ -364,7 +514,7 @@ BTRT_HD FxMoments3 fx_moments3(const fx (&D)[19]) {
 BTRT_HD void fx_expand3(fx a, fx z, fx X, fx Y, fx Z, fx Hx, fx Hy, fx K, fx txy, fx txz, fx tyz, fx (&r)[19]) {
     const fx b = fx_ninth(a) >> 1;                // a / 18
     const fx Hz = -(Hx + Hy), G = (b >> 1) + z - K;
-    r[0] = a - 6 * b - 12 * G;                    // the axis directions sum to 6 b, the diagonals to 12 G
+    r[0] = fx_minus(a - 6 * b, 12 * G);           // the axis directions sum to 6 b, the diagonals to 12 G
     const fx bx = b - Hx, by = b - Hy, bz = b - Hz;
     r[1] = bx + X;
     r[2] = bx - X;
@@ -424,10 +574,8 @@ BTRT_HD bool fx_collide_linear3(const FxFold3 &q, double (&d)[19], double phi_pr
     fx_add(sz, jz, q.Q[5]);
     fx_add(sz, ph, q.P[2]);
     fx_add(sz, pp, q.g[2]);
-    fx a = m.phi;
-    if (!K0ONE) a -= 2 * fx_mul(ph, q.om2);
-    if (SOURCE) a += fx_from<kFxTop3>(src, em);
-    fx r[19];
+    fx a, r[19];
+    if (!fx_density<K0ONE, SOURCE, kFxTop3>(m.phi, ph, q.om2, src, em, a)) return false;
     fx_expand3(a, 0, fx_value(sx), fx_value(sy), fx_value(sz), fx_mul(fx_arg(m.hx), q.d12), fx_mul(fx_arg(m.hy), q.d12),
                fx_mul(fx_arg(m.t3), q.d24), fx_mul(fx_arg(m.pxy), q.d4), fx_mul(fx_arg(m.pxz), q.d4),
                fx_mul(fx_arg(m.pyz), q.d4), r);

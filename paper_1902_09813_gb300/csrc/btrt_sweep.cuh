@@ -631,10 +631,10 @@ __device__ __forceinline__ bool fx_collide_general(const SweepParams<double> &p,
     if constexpr (SRC != kSrcNone) src = src_val * srcv;
     if (SRC != kSrcNone && fx_exp(src) > em + (1u << 20)) return false;
     const fx ks = fx_mul(fx_arg(m.s32), d18), t1 = fx_mul(fx_arg(m.del), d4), t5 = fx_mul(fx_arg(m.pxy), d4);
-    fx a = m.phi, r[9];
+    fx a, r[9];
     const bool k0_one = MODE == kLinearK0One || p.k0_one;
-    if (!k0_one) a -= 2 * fx_mul(fx_arg(m.phi), p.fx.om2);
-    if (SRC != kSrcNone) a += fx_from(src, em);
+    if (k0_one) fx_density<true, SRC != kSrcNone, 58>(m.phi, FxArg{}, p.fx.om2, src, em, a);
+    else if (!fx_density<false, SRC != kSrcNone, 58>(m.phi, fx_arg(m.phi), p.fx.om2, src, em, a)) return false;
     fx_expand(a, z, X, Y, ks, t1, t5, r);
     // the FP64 pipe bounds the per-node coefficients; the constant ones are converted as in
     // fx_collide_linear (ties round differently in the two conversions)

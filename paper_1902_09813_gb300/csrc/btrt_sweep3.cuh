@@ -461,9 +461,9 @@ __device__ __forceinline__ bool fx_collide_general3(const Sweep3Params<double> &
     if constexpr (SRC != kSrcNone) src = p.src_val * srcv;
     if (SRC != kSrcNone && fx_exp(src) > em + (1u << 20)) return false;
     const bool k0_one = MODE == kLinearK0One || p.k0_one;
-    fx a = m.phi, r[19];
-    if (!k0_one) a -= 2 * fx_mul(fx_arg(m.phi), p.fx.om2);
-    if (SRC != kSrcNone) a += fx_from<kFxTop3>(src, em);
+    fx a, r[19];
+    if (k0_one) fx_density<true, SRC != kSrcNone, kFxTop3>(m.phi, FxArg{}, p.fx.om2, src, em, a);
+    else if (!fx_density<false, SRC != kSrcNone, kFxTop3>(m.phi, fx_arg(m.phi), p.fx.om2, src, em, a)) return false;
     fx_expand3(a, z, X, Y, Z, fx_mul(fx_arg(m.hx), d12), fx_mul(fx_arg(m.hy), d12), fx_mul(fx_arg(m.t3), d24),
                fx_mul(fx_arg(m.pxy), d4), fx_mul(fx_arg(m.pxz), d4), fx_mul(fx_arg(m.pyz), d4), r);
     if (k0_one) fx_store<true, 0, kFxTop3>(D, r, p.fx.om2, em, d);
