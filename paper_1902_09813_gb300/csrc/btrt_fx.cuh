@@ -193,11 +193,12 @@ struct FxFold {
     FxConst Qxx, Qxy, Qyy, Px, Py, gx, gy, d18, d4, om2;
     FxConst ux, uy, k06;   // per-node coefficients: u^ and k0/6
     int ok;          // kFxOk* bits; a form whose bit is not set takes the FP64 collision
-    int pad;
+    short hx, hy;    // kFxHalves: u^ is h/2 more than its constant
     double trh, detA;      // half the trace and the determinant of A0^
 };
-// om2, u^ and k0/6 fit; the constant-coefficient form's fit; bgx = bgy; c3 != 0
-enum { kFxOkGeneral = 1, kFxOkLinear = 2, kFxSameB = 4, kFxC3 = 8 };
+// om2, u^ and k0/6 fit; the constant-coefficient form's fit; bgx = bgy; c3 != 0; a
+// component of u^ is a half or more
+enum { kFxOkGeneral = 1, kFxOkLinear = 2, kFxSameB = 4, kFxC3 = 8, kFxHalves = 16 };
 
 // A constant as the products see it.
 inline double fx_real(const FxConst &c) { return ldexp((double)c.hi, -32) + ldexp((double)c.lo, -64); }
@@ -242,7 +243,11 @@ inline bool fx_linear_fits(const FxFold &q) {
 // = 8.3, since K1's eigenvalues lie in (0, 2) and E is tested against 4.
 inline FxFold fx_fold(const double (&Q)[3], const double (&P)[2], const double (&g)[2], double dk, double om,
                       const double (&u)[2], double k0) {
-    const double v[13] = {-Q[0], -Q[1], -Q[2], P[0], P[1], -g[0], -g[1], dk, dk, om, u[0], u[1], k0};
+    // a constant holds less than a half: from there on u^ is split into h/2 and a rest
+    const auto half = [](double t) { return t >= 0.4999 ? 1 : t <= -0.4999 ? -1 : 0; };
+    const int hx = half(u[0]), hy = half(u[1]);
+    const double v[13] = {-Q[0], -Q[1], -Q[2], P[0],           P[1],           -g[0], -g[1],
+                          dk,    dk,    om,    u[0] - 0.5 * hx, u[1] - 0.5 * hy, k0};
     const int div[13] = {6, 6, 6, 6, 6, 6, 6, 18, 4, 2, 1, 1, 6};
     FxConst k[13];
     bool fit[13], lin = true;
@@ -251,9 +256,11 @@ inline FxFold fx_fold(const double (&Q)[3], const double (&P)[2], const double (
         k[i] = fx_const(fit[i] ? v[i] : 0.0, div[i]);
         if (i < 10) lin = lin && fit[i];
     }
-    FxFold q = {k[0], k[1], k[2], k[3], k[4], k[5], k[6], k[7], k[8], k[9], k[10], k[11], k[12], 0, 0, 0.0, 0.0};
+    FxFold q = {k[0], k[1], k[2], k[3], k[4], k[5], k[6], k[7], k[8], k[9], k[10], k[11], k[12], 0, (short)hx, (short)hy, 0.0, 0.0};
     lin = lin && fx_flux_fits(q.Qxx, q.Qxy, q.Px, q.gx) && fx_flux_fits(q.Qxy, q.Qyy, q.Py, q.gy) && fx_linear_fits(q);
-    q.ok = (fit[9] && fit[10] && fit[11] && fit[12] ? kFxOkGeneral : 0) | (lin ? kFxOkLinear : 0);
+    // the low products of k0 j/6 + B's change/6 (up to 15 units) sum below 2^63 up to k0 = 1.9
+    const bool halves = hx || hy, gen = fit[9] && fit[10] && fit[11] && fit[12] && (!halves || k0 < 1.9);
+    q.ok = (gen ? kFxOkGeneral : 0) | (lin ? kFxOkLinear : 0) | (halves ? kFxHalves : 0);
     return q;
 }
 

@@ -36,7 +36,7 @@ namespace btrt {
 
 // A rational constant in the compute type: folded at compile time for
 // float/double, split into its double-word form for dw.
-template <typename Real> __device__ __forceinline__ Real cst(int num, int den) { return Real(num) / Real(den); }
+template <typename Real> BTRT_HD Real cst(int num, int den) { return Real(num) / Real(den); }
 template <> __device__ __forceinline__ dw cst<dw>(int num, int den) { return dw((double)num / (double)den); }
 
 // ---------------------------------------------------------------- storage types
@@ -221,8 +221,8 @@ enum { kSrcNone = 0, kSrcConst = 1, kSrcTrig = 2, kSrcField = 3, kSrcReaction = 
 // max(x, 0)^q for the power-law flux (q != 2) and the reaction term: those
 // terms are defined for phi >= 0, and an undershoot next to a steep front must
 // not turn into a non-finite value.
-__device__ __forceinline__ float powr(float x, float q) { return powf(fmaxf(x, 0.0f), q); }
-__device__ __forceinline__ double powr(double x, double q) { return pow(fmax(x, 0.0), q); }
+BTRT_HD float powr(float x, float q) { return powf(fmaxf(x, 0.0f), q); }
+BTRT_HD double powr(double x, double q) { return pow(fmax(x, 0.0), q); }
 __device__ __forceinline__ dw powr(dw x, dw q) {
     return dw(pow(fmax(static_cast<double>(x), 0.0), static_cast<double>(q)));
 }
@@ -230,14 +230,14 @@ __device__ __forceinline__ dw powr(dw x, dw q) {
 // max(x, 0)^(n + h/2) for a whole or half-whole exponent: n products and one
 // square root (the exponents of Eq. 67 in the paper's tests are 1.5 and 2.5);
 // n < 0 falls back to powr.
-__device__ __forceinline__ float not_negative(float x) { return fmaxf(x, 0.0f); }
-__device__ __forceinline__ double not_negative(double x) { return fmax(x, 0.0); }
+BTRT_HD float not_negative(float x) { return fmaxf(x, 0.0f); }
+BTRT_HD double not_negative(double x) { return fmax(x, 0.0); }
 __device__ __forceinline__ dw not_negative(dw x) { return x.hi > 0.0f ? x : dw(0.0f, 0.0f); }
-__device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
-__device__ __forceinline__ double sqrt_r(double x) { return sqrt(x); }
+BTRT_HD float sqrt_r(float x) { return sqrtf(x); }
+BTRT_HD double sqrt_r(double x) { return sqrt(x); }
 __device__ __forceinline__ dw sqrt_r(dw x) { return dw(sqrt(static_cast<double>(x))); }
 template <typename Real>
-__device__ __forceinline__ Real pow_half(Real x, Real q, int n, int h) {
+BTRT_HD Real pow_half(Real x, Real q, int n, int h) {
     if (n < 0) return powr(x, q);
     const Real xp = not_negative(x);
     Real r = Real(1);
@@ -254,7 +254,7 @@ __device__ __forceinline__ Real flux_pow(const SweepParams<Real> &p, Real phi) {
 
 // Reaction term S = rate phi (1 - phi^exp) (Eq. 67); exp == 2 takes phi phi.
 template <typename Real>
-__device__ __forceinline__ Real reaction(const SweepParams<Real> &p, Real phi) {
+BTRT_HD Real reaction(const SweepParams<Real> &p, Real phi) {
     const Real pe = p.react2 ? phi * phi : pow_half(phi, p.react_exp, p.re_n, p.re_h);
     return p.react_rate * phi * (Real(1) - pe);
 }
@@ -497,9 +497,13 @@ static __device__ __noinline__ double collide_f64_slow_own(const SweepParams<dou
 // 1/v by Householder's third-order iteration on the hardware's approximate
 // reciprocal (relative error e below 2^-18): x (1 + e + e^2), error e^3 plus the
 // rounding of the last step.
-__device__ __forceinline__ double recip_f64(double v) {
+BTRT_HD double recip_f64(double v) {
     double x;
+#ifdef __CUDA_ARCH__
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(v));
+#else
+    x = fx_double(fx_bits(1.0 / v) & ~0x1ffffffffull);   // host tests: a seed cut to 20 bits
+#endif
     const double e = fma(-v, x, 1.0);
     return fma(x, fma(e, e, e), x);
 }
@@ -510,7 +514,7 @@ __device__ __forceinline__ double recip_f64(double v) {
 // share one reciprocal).  Returns false, with d untouched, when a value leaves
 // the integer form's range.
 template <int MODE, int SRC>
-__device__ __forceinline__ bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], double phi_prev,
+BTRT_HD bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], double phi_prev,
                                                    double srcv, int node, double src_val, double &phi_out) {
     const FoldConsts<double> &L = p.lin;
     unsigned int em;
@@ -545,8 +549,15 @@ __device__ __forceinline__ bool fx_collide_general(const SweepParams<double> &p,
         const unsigned int far = em + (1u << 20);
         if (fx_exp(gsx) > far || fx_exp(gsy) > far || fx_exp(gdx) > far || fx_exp(gdy) > far) return false;
         const FxArg mean = fx_arg((m.phi + pv) >> 1), diff = fx_arg(m.phi - pv);
-        const fx Ex = fx_mul(mean, p.fx.ux) + fx_from(gsx, em) - m.jx, Ey = fx_mul(mean, p.fx.uy) + fx_from(gsy, em) - m.jy;
-        const fx Dx = fx_mul(diff, p.fx.ux) + fx_from(gdx, em), Dy = fx_mul(diff, p.fx.uy) + fx_from(gdy, em);
+        fx Ex = fx_mul(mean, p.fx.ux) + fx_from(gsx, em) - m.jx, Ey = fx_mul(mean, p.fx.uy) + fx_from(gsy, em) - m.jy;
+        fx Dx = fx_mul(diff, p.fx.ux) + fx_from(gdx, em), Dy = fx_mul(diff, p.fx.uy) + fx_from(gdy, em);
+        if (p.fx.ok & kFxHalves) {
+            const fx mh = (m.phi + pv) >> 2, dh = (m.phi - pv) >> 1;
+            Ex += p.fx.hx * mh;
+            Ey += p.fx.hy * mh;
+            Dx += p.fx.hx * dh;
+            Dy += p.fx.hy * dh;
+        }
         const double p2 = phi * phi;
         if (p.fx.ok & kFxC3) {
             // C(phi) - phi: in sigma, and k0 (C - phi) / 18 in the isotropic terms

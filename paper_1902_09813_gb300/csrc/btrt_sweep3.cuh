@@ -351,14 +351,14 @@ static __device__ __noinline__ void init3_f64_slow(const Sweep3Params<double> &p
     for (int i = 0; i < 19; ++i) t[i] = fma(wgt3<double>(i), src, d[i]);
 }
 
-__device__ __forceinline__ double reaction3(const Sweep3Params<double> &p, double phi) {
+BTRT_HD double reaction3(const Sweep3Params<double> &p, double phi) {
     return p.react_rate * phi * (1.0 - (p.react2 ? phi * phi : pow_half(phi, p.react_exp, p.re_n, p.re_h)));
 }
 
 // Per-node coefficients or a reaction source: integer moments and populations, FP64
 // coefficients and V.
 template <int MODE, int SRC>
-__device__ __forceinline__ bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19], double phi_prev,
+BTRT_HD bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19], double phi_prev,
                                                     double srcv, double &phi_out) {
     unsigned int em;
     if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;

@@ -74,3 +74,12 @@ def test_equal_populations_d3q19(kind, k0):
     field = 3 * 1.99 / 64 * np.array([1.0, 6.0, 12.0, 12.0])[n]
     p = _with(p.replace(A0=(a, 0.0, 0.0, a, 0.0, a), phi0_fn=lambda X, Y, Z: field), kind, k0)
     _check3(p, 2)
+
+
+@pytest.mark.parametrize("u", [(0.45, 0.52), (-0.55, 0.3), (0.7, -0.95)], ids=str)
+@pytest.mark.parametrize("k0", [1.0, 1.2])
+@pytest.mark.parametrize("size", [(41, 33), (37, 29)], ids=["many-steps", "plain"])
+def test_fast_flow(u, k0, size):
+    """Per-node coefficients with half a cell and more per step."""
+    p = w.random_state_problem(*size, seed=4, bc=(0, 0, 1, 1), nonlinear=True, source="trig").replace(u=u, k0=k0)
+    _check2(p, (5,))
