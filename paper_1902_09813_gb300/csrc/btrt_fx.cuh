@@ -16,9 +16,9 @@
 // to 2^-53.  The four-times-smaller axis populations and the sixteen-times-smaller
 // diagonal ones keep errors at or below those of the FP64 form; their sum is exact
 // (r_0 is formed as the total minus the other eight).
-// Range: exponents 64 .. 2040 (about 1e-289 .. 1e306); below it a result is the
-// nearest multiple of 2^-1017, above it (and for infinities and NaN) the node takes
-// the FP64 form (collide_f64_slow).
+// Range: largest populations of exponent 64 .. 2040 (about 1e-289 .. 1e306), or nodes that
+// are zero throughout; the others (and infinities and NaN) take the FP64 form
+// (collide_f64_slow).
 #pragma once
 
 #include <math.h>
@@ -326,15 +326,34 @@ BTRT_HD FxMoments fx_moments(const fx (&D)[9]) {
     return m;
 }
 
-// The common exponent of a node's populations; false when it leaves the range.
+// The common exponent of a node's populations; false outside the range.
 template <int N> BTRT_HD bool fx_common_exp(const double (&d)[N], unsigned int &em) {
-    em = kFxExpMin;
+    em = fx_exp(d[0]);
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
+    for (int i = 1; i < N; ++i) {
         const unsigned int e = fx_exp(d[i]);
         em = em > e ? em : e;
     }
-    return em <= kFxExpMax;
+    return em - kFxExpMin <= kFxExpMax - kFxExpMin;
+}
+
+// Whether a node is zero throughout (its results then are as well).
+BTRT_HD bool fx_all_zero(const double *d, int n, double phi_prev, double src) {
+    unsigned long long any = fx_bits(phi_prev) | fx_bits(src);
+    for (int i = 0; i < n; ++i) any |= fx_bits(d[i]);
+    return (any << 1) == 0;
+}
+// A node whose largest population is out of the range: large values take the FP64 form, and
+// so do tiny ones, for its gradual underflow; zeros are done.  On the device the
+// out-of-line FP64 forms look for those: with the test in line the 8192^2 sweep took
+// 38.56 ms instead of 37.48.
+template <int N> BTRT_HD bool fx_out_of_range(const double (&d)[N], double phi_prev, double src, double &phi_out) {
+#ifdef __CUDA_ARCH__
+    return false;
+#else
+    phi_out = 0.0;
+    return fx_all_zero(d, N, phi_prev, src);
+#endif
 }
 
 // The outputs of a node, (1 - k0) D_i + r_i, as FP64; the first NADD by the FP64
@@ -364,7 +383,8 @@ BTRT_HD void fx_store(const fx (&D)[N], const fx (&r)[N], const FxConst &om2, un
 template <bool K0ONE, bool SOURCE>
 BTRT_HD bool fx_collide_linear(const FxFold &q, double (&d)[9], double phi_prev, double src, double &phi_out) {
     unsigned int em;
-    if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;
+    if (!fx_common_exp(d, em)) return fx_out_of_range(d, phi_prev, SOURCE ? src : 0.0, phi_out);
+    if (fx_exp(phi_prev) > em + (2u << 20)) return false;
     if (SOURCE && fx_exp(src) > em + (1u << 20)) return false;
     fx D[9];
 #pragma unroll
@@ -557,7 +577,8 @@ BTRT_HD void fx_expand3(fx a, fx z, fx X, fx Y, fx Z, fx Hx, fx Hy, fx K, fx txy
 template <bool K0ONE, bool SOURCE>
 BTRT_HD bool fx_collide_linear3(const FxFold3 &q, double (&d)[19], double phi_prev, double src, double &phi_out) {
     unsigned int em;
-    if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;
+    if (!fx_common_exp(d, em)) return fx_out_of_range(d, phi_prev, SOURCE ? src : 0.0, phi_out);
+    if (fx_exp(phi_prev) > em + (2u << 20)) return false;
     if (SOURCE && fx_exp(src) > em + (1u << 20)) return false;
     fx D[19];
 #pragma unroll

@@ -477,6 +477,7 @@ __device__ __forceinline__ double collide_f64_plain(const SweepParams<double> &p
     double d[9], phid;
 #pragma unroll
     for (int i = 0; i < 9; ++i) d[i] = t[i];
+    if (fx_all_zero(d, 9, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv)) return 0.0;
     const double phi =
         collide_fold<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, node, phid, nullptr, sv);
 #pragma unroll
@@ -518,7 +519,8 @@ BTRT_HD bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], do
                                                    double srcv, int node, double src_val, double &phi_out) {
     const FoldConsts<double> &L = p.lin;
     unsigned int em;
-    if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;
+    if (!fx_common_exp(d, em)) return fx_out_of_range(d, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv, phi_out);
+    if (fx_exp(phi_prev) > em + (2u << 20)) return false;
     fx D[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) D[i] = fx_from(d[i], em);
@@ -672,9 +674,10 @@ __device__ __forceinline__ void init_f64(const SweepParams<double> &p, double (&
         Cm = p.c3 * phi * phi * phi;
     }
     unsigned int em = fx_exp(phi);
+    const bool tiny = em < kFxExpMin && ((fx_bits(phi) | fx_bits(src)) << 1) != 0;
     em = em > kFxExpMin ? em : kFxExpMin;
     const unsigned int far = em + (1u << 20);
-    if (em > kFxExpMax || fx_exp(Bx) > far || fx_exp(By) > far || fx_exp(src) > far || fx_exp(Cm) > far) {
+    if (tiny || em > kFxExpMax || fx_exp(Bx) > far || fx_exp(By) > far || fx_exp(src) > far || fx_exp(Cm) > far) {
         double t[9];
         init_f64_slow<MODE, SRC>(p, t, phi, src);
 #pragma unroll

@@ -339,6 +339,7 @@ static __device__ __noinline__ double collide3_f64_slow(const Sweep3Params<doubl
     double d[19], phid;
 #pragma unroll
     for (int i = 0; i < 19; ++i) d[i] = t[i];
+    if (fx_all_zero(d, 19, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv)) return 0.0;
     const double phi = collide3<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, phid);
 #pragma unroll
     for (int i = 0; i < 19; ++i) t[i] = d[i];
@@ -361,7 +362,8 @@ template <int MODE, int SRC>
 BTRT_HD bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19], double phi_prev,
                                                     double srcv, double &phi_out) {
     unsigned int em;
-    if (!fx_common_exp(d, em) || fx_exp(phi_prev) > em + (2u << 20)) return false;
+    if (!fx_common_exp(d, em)) return fx_out_of_range(d, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv, phi_out);
+    if (fx_exp(phi_prev) > em + (2u << 20)) return false;
     fx D[19];
 #pragma unroll
     for (int i = 0; i < 19; ++i) D[i] = fx_from<kFxTop3>(d[i], em);
@@ -484,9 +486,10 @@ __device__ __forceinline__ void init3_f64(const Sweep3Params<double> &p, double 
         Cm = p.c3 * phi * phi * phi;
     }
     unsigned int em = fx_exp(phi);
+    const bool tiny = em < kFxExpMin && ((fx_bits(phi) | fx_bits(src)) << 1) != 0;
     em = em > kFxExpMin ? em : kFxExpMin;
     const unsigned int far = em + (1u << 20);
-    if (em > kFxExpMax || fx_exp(Bx) > far || fx_exp(By) > far || fx_exp(Bz) > far || fx_exp(src) > far ||
+    if (tiny || em > kFxExpMax || fx_exp(Bx) > far || fx_exp(By) > far || fx_exp(Bz) > far || fx_exp(src) > far ||
         fx_exp(Cm) > far) {
         double t[19];
         init3_f64_slow(p, t, phi, src);

@@ -106,3 +106,28 @@ def test_ordinary_states_are_not_refused(lib, dim):
             assert _node(lib, v, d, prev, 0.1 * src, 1)[0] == 1
             full = [float(w) * (1 + 0.1 * rng.uniform(-1, 1)) for w in WGT[dim]]
             assert _node(lib, v, full, 1.0, 0.1, 1)[0] == 1
+
+
+@pytest.mark.parametrize("k0", [1.0, 1.1])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_tiny_nodes_are_left_to_fp64(lib, dim, k0):
+    """Below 2^-959 the integers' unit would be coarser than FP64's own: such nodes are refused
+    with the populations untouched; a node of zeros is not."""
+    v = _coeffs(np.random.default_rng(1), k0, dim)
+    Q = len(VEL[dim])
+    for e in (-965, -1000, -1030, -1070):
+        d = [float(t) * 2.0 ** e for t in WGT[dim]]
+        ok, got, _ = _node(lib, v, d, 2.0 ** e, 0.0, 0)
+        assert ok == 0 and got == d
+        for k in range(Q):
+            one = [0.0] * Q
+            one[k] = -(2.0 ** e)
+            ok, got, _ = _node(lib, v, one, 0.0, 0.0, 0)
+            assert ok == 0 and got == one
+        assert _node(lib, v, [0.0] * Q, 2.0 ** e, 0.0, 1)[0] == 0
+        assert _node(lib, v, [0.0] * Q, 0.0, -(2.0 ** e), 1)[0] == 0
+    for z in (0.0, -0.0):
+        ok, got, phi = _node(lib, v, [z] * Q, z, z, 1)
+        assert ok == 1 and got == [0.0] * Q and phi == 0.0
+    d = [float(t) * 2.0 ** -955 for t in WGT[dim]]
+    assert _node(lib, v, d, 2.0 ** -955, 0.0, 0)[0] == 1

@@ -83,3 +83,25 @@ def test_fast_flow(u, k0, size):
     """Per-node coefficients with half a cell and more per step."""
     p = w.random_state_problem(*size, seed=4, bc=(0, 0, 1, 1), nonlinear=True, source="trig").replace(u=u, k0=k0)
     _check2(p, (5,))
+
+
+@pytest.mark.parametrize("nonlinear", [False, True])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_tiny_values(dim, nonlinear):
+    """A field around 1e-300, with zeros: the relative accuracy of ordinary values."""
+    n, draw = ((48, 37), w.random_state_problem) if dim == 2 else ((12, 11, 9), w.random_state_problem3)
+    p = draw(*n, seed=6, nonlinear=nonlinear, source="none")
+    field = 1e-300 * p.phi0()
+    field[..., :5] = 0.0
+    if dim == 2:
+        from paper_1902_09813_gb300 import Lattice as L
+        ref = oracle.OracleLattice(p.replace(phi0_array=field), nthreads=cpu_threads()).init()
+    else:
+        from paper_1902_09813_gb300 import Lattice3 as L
+        ref = o3.OracleLattice3(p.replace(phi0_fn=lambda X, Y, Z: field), nthreads=cpu_threads()).init()
+    lat = L.from_problem(p, compute="f64").init(field).step(3)
+    ref.step(3)
+    assert lat.check() == 0
+    assert _rel(lat.phi_host() * 2.0 ** 990, ref.phi() * 2.0 ** 990) <= TOL64
+    ref.step(1)
+    assert _rel(lat.read_f() * 2.0 ** 990, ref.fpost * 2.0 ** 990) <= TOL64
