@@ -91,7 +91,7 @@ FP64_NOMINAL_TOPS = 0.625
 # to them both are re-taken and the digest updated (a CPU test checks it), and
 # until then the traffic is reported as null.
 FP64_SWEEP_SOURCES = ("btrt_sweep.cuh", "btrt_dw.cuh", "btrt_fx.cuh")   # the FP64 sweep's device code
-FP64_SWEEP_DIGEST = "74aaf7b9ed05c7dd"
+FP64_SWEEP_DIGEST = "456b9cbfc32ac90b"
 FP64_TRAFFIC_PER_NODE = 148.2
 # DRAM bytes per node and step of the two-step FP32-compute kernel measured by ncu,
 # keyed by (storage, shift), for the sources with digest TB2_DIGEST.

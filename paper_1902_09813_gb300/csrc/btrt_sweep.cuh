@@ -503,7 +503,8 @@ BTRT_HD double recip_f64(double v) {
 #ifdef __CUDA_ARCH__
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(v));
 #else
-    x = fx_double(fx_bits(1.0 / v) & ~0x1ffffffffull);   // host tests: a seed cut to 20 bits
+    x = 1.0 / v;   // host tests: a seed cut to 20 bits, subnormals flushed as the hardware does
+    x = fx_exp(x) == 0 ? 0.0 : fx_double(fx_bits(x) & ~0x1ffffffffull);
 #endif
     const double e = fma(-v, x, 1.0);
     return fma(x, fma(e, e, e), x);

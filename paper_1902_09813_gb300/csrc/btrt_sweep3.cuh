@@ -418,6 +418,7 @@ BTRT_HD bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19],
             id = recip_f64(det);
             k2 = p.k2c;
         }
+        if (fx_exp(id) == 0) return false;   // the reciprocal underflowed (and k2 with it)
         const double dk = k2 - p.k0;
         // K1 e with the cofactors, divided by the determinant once per component
         const double ex = id * fma(-0.5, dBx, Bx - jx), ey = id * fma(-0.5, dBy, By - jy), ez = id * fma(-0.5, dBz, Bz - jz);

@@ -215,6 +215,31 @@ def test_errors_no_larger_than_plain_fp64(lib, dim, k0):
     assert (e[0] <= e[1]).all(), np.sqrt(e / n)
 
 
+@pytest.mark.parametrize("k2", [-1.0, 0.7])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_coefficients_past_the_reciprocal(lib, dim, k2):
+    """Diffusivities so large that the shared reciprocal 1/(det ..) underflows: right or refused."""
+    rng = np.random.default_rng(9)
+    c = _coeffs(rng, dim, 2.0, 0.0, 1.0, k2, 0.0, 0.1)
+    A = [0.05 if a == b else 0.0 for a in range(dim) for b in range(a, dim)]
+    c[2 * dim + 2:-5] = A
+    d, prev = _state(rng, dim)
+    powers = np.arange(230.0, 520.0, 0.25)
+    taken = 0
+    for e in powers:
+        c[-5] = float(2.0 ** e)
+        t = list(d)
+        ok, got, phi = _node(lib, c, t, prev)
+        taken += ok
+        if ok != 1:
+            assert got == d
+            continue
+        ref, _, _ = _collide(c, d, prev, Decimal, dim)
+        for g, r in zip(got, ref):
+            assert abs(Decimal(g) - r) <= Decimal("1e-14")
+    assert 0 < taken < len(powers)
+
+
 def test_reciprocal(lib):
     """Householder's iteration leaves the cube of the seed's error (2^-57 and less) and the rounding
     of its last step."""
