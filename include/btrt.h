@@ -233,9 +233,15 @@ btrt_status btrt_check(btrt_lattice L, int32_t *flags);
  * _TB2V: BTRT_EINVAL). */
 enum {
     BTRT_SWEEP_AUTO = 0, BTRT_SWEEP_PLAIN = 1, BTRT_SWEEP_TMA = 2, BTRT_SWEEP_TB2 = 3, BTRT_SWEEP_VEC = 4,
-    BTRT_SWEEP_TB2V = 5
+    BTRT_SWEEP_TB2V = 5, BTRT_SWEEP_MANY = 6
 };
 btrt_status btrt_set_sweep_variant(btrt_lattice L, int32_t variant);
+
+/* The form that BTRT_SWEEP_AUTO takes for btrt_step of two steps or more on such a
+ * lattice: BTRT_SWEEP_MANY (many steps per launch; only ever AUTO's choice),
+ * _TB2, _VEC or _PLAIN.  per_node: the coefficients are evaluated per node (b2, c3 or a2
+ * not zero, or a diffusion field).  Touches no device. */
+btrt_status btrt_auto_form(const btrt_grid_desc *desc, int32_t per_node, int32_t *form);
 
 /* Number of completed steps and the current time t0 + n dt. */
 btrt_status btrt_get_time(btrt_lattice L, int64_t *step, double *t);

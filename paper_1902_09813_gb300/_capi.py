@@ -13,7 +13,7 @@ F64, F32, F16, BF16, DF64 = 0, 1, 2, 3, 4
 K2_HBB, K2_CONST = 0, 1
 SRC_NONE, SRC_CONST, SRC_TRIG, SRC_FIELD, SRC_REACTION = 0, 1, 2, 3, 4
 FIELD_SOURCE, FIELD_DIFFUSION = 1, 2
-SWEEP_AUTO, SWEEP_PLAIN, SWEEP_TMA, SWEEP_TB2, SWEEP_VEC, SWEEP_TB2V = 0, 1, 2, 3, 4, 5
+SWEEP_AUTO, SWEEP_PLAIN, SWEEP_TMA, SWEEP_TB2, SWEEP_VEC, SWEEP_TB2V, SWEEP_MANY = 0, 1, 2, 3, 4, 5, 6
 SHIFT_REF, SHIFT_LOCAL = 0, 1
 PROBE_FMA, PROBE_ADD, PROBE_MUL = 0, 1, 2
 SHIFT_LOCAL_DW, SHIFT_LOCAL_SR, SHIFT_LOCAL_DW_SR, SHIFT_MOMENT_SR = 2, 3, 4, 5
@@ -96,6 +96,7 @@ SIGNATURES = [
     ("btrt_mass", ctypes.c_int, [_vp, _dp]),
     ("btrt_check", ctypes.c_int, [_vp, ctypes.POINTER(_i32)]),
     ("btrt_set_sweep_variant", ctypes.c_int, [_vp, _i32]),
+    ("btrt_auto_form", ctypes.c_int, [ctypes.POINTER(GridDesc), _i32, ctypes.POINTER(_i32)]),
     ("btrt_get_time", ctypes.c_int, [_vp, ctypes.POINTER(_i64), _dp]),
     ("btrt_state_bytes", _sz, [_vp]),
     ("btrt_save", ctypes.c_int, [_vp, _vp, _sz]),

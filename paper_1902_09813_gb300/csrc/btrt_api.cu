@@ -413,17 +413,60 @@ constexpr long long kVecAutoNodes = 1LL << 21;
 // us per step, vector / plain, 800^2 16.7 / 15.2, 900^2 17.4 / 17.5, 1024^2 19.4 / 21.3 (FP16
 // 25.5 / 25.6, nonlinear BF16 24.6 / 21.5).
 constexpr long long kVecMomentNodes = 7LL << 17;
-int btrt::effective_sweep_variant(btrt_lattice L) {
-    if (L->g.compute != BTRT_F32 || has_phi_lo(L->g)) return BTRT_SWEEP_PLAIN;
-    if (L->sweep_variant != BTRT_SWEEP_AUTO) return L->sweep_variant;
-    const bool s16 = L->g.storage == BTRT_F16 || L->g.storage == BTRT_BF16;
-    const bool large = (long long)L->g.nx * L->g.ny >= kVecAutoNodes;
-    if (stochastic_store(L->g)) {
-        const bool moment = has_j(L->g) && L->g.storage == BTRT_BF16 && sweep_mode(L) != kGeneral &&
-                            (long long)L->g.nx * L->g.ny >= kVecMomentNodes;
+static int auto_step_form(const btrt_grid_desc &g, bool general) {
+    if (g.compute != BTRT_F32 || has_phi_lo(g)) return BTRT_SWEEP_PLAIN;
+    const bool s16 = g.storage == BTRT_F16 || g.storage == BTRT_BF16;
+    const bool large = (long long)g.nx * g.ny >= kVecAutoNodes;
+    if (stochastic_store(g)) {
+        const bool moment = has_j(g) && g.storage == BTRT_BF16 && !general && (long long)g.nx * g.ny >= kVecMomentNodes;
         return large || moment ? BTRT_SWEEP_VEC : BTRT_SWEEP_PLAIN;
     }
     return s16 && large ? BTRT_SWEEP_VEC : BTRT_SWEEP_TB2;
+}
+int btrt::effective_sweep_variant(btrt_lattice L) {
+    if (L->g.compute != BTRT_F32 || has_phi_lo(L->g)) return BTRT_SWEEP_PLAIN;
+    if (L->sweep_variant != BTRT_SWEEP_AUTO) return L->sweep_variant;
+    return auto_step_form(L->g, sweep_mode(L) == kGeneral);
+}
+
+// Whether AUTO advances a lattice many steps per launch (btrt_tbn.cuh): sides of at
+// least one region width, and few enough nodes.  Measured us per step, many steps per
+// launch against the form AUTO takes otherwise (square lattices, 200 steps with set-up
+// and read): FP32 storage 64^2 1.7 / 5.2, 256^2 2.6 / 5.2, 362^2 3.8 / 5.3, 430^2 5.7 / 5.3;
+// FP16 local shift 64^2 1.8 / 6.3, 362^2 3.9 / 6.3, 512^2 6.5 / 7.3 (nonlinear 6.8 / 9.4);
+// double-word phi 512^2 6.6 / 10.4, with constant coefficients 540^2 8.4 / 10.4, 640^2
+// 10.9 / 12.5, 724^2 10.9 / 13.2; first-moment form 512^2 7.8 / 10.4; FP64 hill 64^2 2.1 / 6.3,
+// 160^2 3.1 / 6.3, 181^2 5.0 / 6.3, 256^2 6.9 / 6.3, nonlinear 160^2 10.2 / 12.3, 181^2
+// 14.8 / 12.4; double-word format hill 256^2 6.1 / 6.3, nonlinear 181^2 6.2 / 6.3.
+//
+// Lattices of up to 2^18 nodes make more tiles than are resident (28 x 8 nodes each at depth 2,
+// four 256-thread blocks on each of 152 SMs), and narrow ones most: this form's time goes
+// with the waves of tiles, that of the others with their 32-node columns.  So the waves after
+// the first have to be worth it, by the nodes of those columns.  us per step of 120 steps,
+// other form / this one.  FP16 local shift, third wave: hill 32 x 7776 9.4 / 11.4, 57 x 3400
+// 7.9 / 8.5, 57 x 3888 9.1 / 8.5, 100 x 2552 10.6 / 8.7, nonlinear 32 x 8192 8.2 / 11.1, 100 x 2552 9.2 / 8.5;
+// second wave, nonlinear 32 x 2672 6.2 / 6.0, front 64 x 3160 10.3 / 9.2.  Rounded stochastically, hill 32 x 5104
+// 8.2 / 8.0 (first-moment form 8.2 / 9.2), 64 x 3400 8.2 / 8.0 (10.3 / 9.1); nonlinear, second wave
+// 32 x 2672 6.2 / 6.7 (6.2 / 7.4), 128 x 1064 7.1 / 6.6 (8.2 / 7.4), third 64 x 3400 8.2 / 9.6 (10.3 / 10.7),
+// 57 x 4536 10.3 / 9.8 (12.3 / 11.0); front, second 57 x 1776 8.2 / 9.6 (8.2 / 10.5), third 128 x 2040
+// 10.9 / 13.3 (12.2 / 14.6).  FP32 storage ends within two waves (0.95 to 1.5 times the two-step form's
+// rate over widths 32 to 200); double-word phi stays ahead through three (nonlinear) or six
+// (constant coefficients).
+constexpr long long kTbnResident = 4 * 152;
+static bool takes_many_steps(const btrt_grid_desc &g, bool general) {
+    if (g.nx < 32 || g.ny < 32) return false;
+    const long long nodes = (long long)g.nx * g.ny;
+    if (g.compute == BTRT_F64) return nodes <= (general ? 3 << 13 : 1 << 15);
+    if (g.compute == BTRT_DF64) return nodes <= (general ? 1 << 15 : 1 << 16);
+    if (g.storage == BTRT_F32 && !has_phi_lo(g)) return nodes <= 1 << 17;
+    if (g.storage == BTRT_F32 && !general) return nodes <= 1 << 19;
+    const long long tiles = (long long)((g.nx + 27) / 28) * ((g.ny + 7) / 8);
+    const long long waves = (tiles + kTbnResident - 1) / kTbnResident;
+    const long long columns = (long long)((g.nx + 31) / 32) * 32 * g.ny;
+    if (nodes > 1 << 18 || waves > 3) return false;
+    if (general && stochastic_store(g)) return columns >= (waves - 1) << 17;
+    if (waves <= 2 || (has_phi_lo(g) && !stochastic_store(g))) return true;
+    return columns >= (stochastic_store(g) ? 3 << 16 : 15 << 14);
 }
 
 namespace {
@@ -455,25 +498,8 @@ btrt_status launch(btrt_lattice L, int64_t n, bool first, bool resid = false) {
     return BTRT_OK;
 }
 
-// Whether btrt_step advances L many steps per launch (btrt_tbn.cuh): AUTO, sides of at
-// least one region width, and few enough nodes.  Measured us per step, many steps per
-// launch against the form AUTO takes otherwise (square lattices, 200 steps with set-up
-// and read): FP32 storage 64^2 1.7 / 5.2, 256^2 2.6 / 5.2, 362^2 3.8 / 5.3, 430^2 5.7 / 5.3;
-// FP16 local shift 64^2 1.8 / 6.3, 362^2 3.9 / 6.3, 512^2 6.5 / 7.3 (nonlinear 6.8 / 9.4);
-// double-word phi 512^2 6.6 / 10.4, with constant coefficients 540^2 8.4 / 10.4, 640^2
-// 10.9 / 12.5, 724^2 10.9 / 13.2; first-moment form 512^2 7.8 / 10.4; FP64 hill 64^2 2.1 / 6.3,
-// 160^2 3.1 / 6.3, 181^2 5.0 / 6.3, 256^2 6.9 / 6.3, nonlinear 160^2 10.2 / 12.3, 181^2
-// 14.8 / 12.4; double-word format hill 256^2 6.1 / 6.3, nonlinear 181^2 6.2 / 6.3.
 bool takes_tbn(btrt_lattice L) {
-    const btrt_grid_desc &g = L->g;
-    if (L->sweep_variant != BTRT_SWEEP_AUTO || g.nx < 32 || g.ny < 32) return false;
-    const bool general = sweep_mode(L) == kGeneral;
-    long long most;
-    if (g.compute == BTRT_F64) most = general ? 3 << 13 : 1 << 15;
-    else if (g.compute == BTRT_DF64) most = general ? 1 << 15 : 1 << 16;
-    else if (g.storage == BTRT_F32 && !has_phi_lo(g)) most = 1 << 17;
-    else most = g.storage == BTRT_F32 && !general ? 1 << 19 : 1 << 18;
-    return (long long)g.nx * g.ny <= most;
+    return L->sweep_variant == BTRT_SWEEP_AUTO && takes_many_steps(L->g, sweep_mode(L) == kGeneral);
 }
 
 template <typename Real>
@@ -1032,6 +1058,14 @@ btrt_status btrt_set_sweep_variant(btrt_lattice L, int32_t variant) {
     if (variant == BTRT_SWEEP_TMA && !L->have_tma)
         return fail(BTRT_EINVAL, "the TMA sweep serves FP32-compute lattices whose tensor maps could be encoded");
     L->sweep_variant = variant;
+    return BTRT_OK;
+}
+
+btrt_status btrt_auto_form(const btrt_grid_desc *desc, int32_t per_node, int32_t *form) {
+    if (!form) return fail(BTRT_EINVAL, "null argument");
+    btrt_status st = check_desc(desc);
+    if (st != BTRT_OK) return st;
+    *form = takes_many_steps(*desc, per_node != 0) ? BTRT_SWEEP_MANY : auto_step_form(*desc, per_node != 0);
     return BTRT_OK;
 }
 

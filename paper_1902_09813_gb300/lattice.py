@@ -60,6 +60,14 @@ def workspace_bytes(desc: C.GridDesc) -> int:
     return int(n)
 
 
+def auto_form(desc: C.GridDesc, per_node: bool) -> str:
+    """The kernel form that 'auto' takes for two or more steps of such a lattice: 'many' (many
+    steps per launch), 'tb2', 'vec' or 'plain' (see btrt_auto_form in include/btrt.h)."""
+    form = ctypes.c_int32()
+    C.check(C.load().btrt_auto_form(ctypes.byref(desc), 1 if per_node else 0, ctypes.byref(form)))
+    return {C.SWEEP_MANY: "many", C.SWEEP_TB2: "tb2", C.SWEEP_VEC: "vec", C.SWEEP_PLAIN: "plain"}[form.value]
+
+
 def batch_workspace_bytes(descs) -> int:
     """Device bytes of the batch tables for lattices with these grid descriptions."""
     arr = (C.GridDesc * len(descs))(*descs)
