@@ -502,8 +502,11 @@ bool takes_tbn(btrt_lattice L) {
     return L->sweep_variant == BTRT_SWEEP_AUTO && takes_many_steps(L->g, sweep_mode(L) == kGeneral);
 }
 
+// n steps in one launch; *taken = false, with nothing done, when the launch is refused
+// because its blocks are not all resident at once: the context has fewer SMs than the
+// device the grid is sized for.
 template <typename Real>
-btrt_status launch_tbn(btrt_lattice L, int n) {
+btrt_status launch_tbn(btrt_lattice L, int n, bool *taken) {
     SweepParams<Real> p;
     fill_params(L, p, L->step + 1, false);
     TbnSteps<Real> st;
@@ -519,11 +522,18 @@ btrt_status launch_tbn(btrt_lattice L, int n) {
     }
     const int mode = sweep_mode(L), sh = shift_of(L->g);
     int rounds = 0;   // one buffer flip each
-    if constexpr (std::is_same<Real, double>::value) CUDA_TRY(launch_sweep_tbn_f64(p, st, mode, &rounds, L->stream));
-    else if constexpr (std::is_same<Real, dw>::value) CUDA_TRY(launch_sweep_tbn_dw(p, st, mode, &rounds, L->stream));
-    else if (L->g.storage == BTRT_F32) CUDA_TRY(launch_sweep_tbn_f32(p, st, sh, mode, &rounds, L->stream));
-    else if (L->g.storage == BTRT_F16) CUDA_TRY(launch_sweep_tbn_f16(p, st, sh, mode, &rounds, L->stream));
-    else CUDA_TRY(launch_sweep_tbn_bf16(p, st, sh, mode, &rounds, L->stream));
+    cudaError_t e;
+    if constexpr (std::is_same<Real, double>::value) e = launch_sweep_tbn_f64(p, st, mode, &rounds, L->stream);
+    else if constexpr (std::is_same<Real, dw>::value) e = launch_sweep_tbn_dw(p, st, mode, &rounds, L->stream);
+    else if (L->g.storage == BTRT_F32) e = launch_sweep_tbn_f32(p, st, sh, mode, &rounds, L->stream);
+    else if (L->g.storage == BTRT_F16) e = launch_sweep_tbn_f16(p, st, sh, mode, &rounds, L->stream);
+    else e = launch_sweep_tbn_bf16(p, st, sh, mode, &rounds, L->stream);
+    *taken = e != cudaErrorCooperativeLaunchTooLarge;
+    if (!*taken) {
+        cudaGetLastError();
+        return BTRT_OK;
+    }
+    CUDA_TRY(e);
     L->cur = (L->cur + rounds) & 1;
     L->step += n;
     return BTRT_OK;
@@ -885,10 +895,12 @@ btrt_status btrt_step(btrt_lattice L, int64_t nsteps) {
     if (takes_tbn(L))
         while (nsteps >= 2) {
             const int n = (int)std::min<int64_t>(nsteps, kTbnMaxSteps);
-            btrt_status st = L->g.compute == BTRT_F64    ? launch_tbn<double>(L, n)
-                             : L->g.compute == BTRT_DF64 ? launch_tbn<dw>(L, n)
-                                                         : launch_tbn<float>(L, n);
+            bool taken = false;
+            btrt_status st = L->g.compute == BTRT_F64    ? launch_tbn<double>(L, n, &taken)
+                             : L->g.compute == BTRT_DF64 ? launch_tbn<dw>(L, n, &taken)
+                                                         : launch_tbn<float>(L, n, &taken);
             if (st != BTRT_OK) return st;
+            if (!taken) break;   // the forms below take the rest
             nsteps -= n;
         }
     // the two-step forms serve every FP32-compute lattice (AUTO: see effective_sweep_variant)

@@ -1,0 +1,55 @@
+"""Many steps per launch: what its cooperative launch does when it is refused."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+from conftest import ROOT
+
+pytestmark = pytest.mark.gpu
+
+# cudaLaunchCooperativeKernel that answers cudaErrorCooperativeLaunchTooLarge and launches nothing
+FAKE = r"""
+#include <stdio.h>
+int cudaLaunchCooperativeKernel(const void *f, ...) {
+    (void)f;
+    fprintf(stderr, "refused\n");
+    return 720;
+}
+"""
+RUN = r"""
+import sys
+sys.path[:0] = [%r, %r]
+import numpy as np
+import workloads as w
+from paper_1902_09813_gb300 import Lattice
+for form in (("f64", "f64", "ref"), ("df64", "df64", "ref"), ("f32", "f32", "ref"), ("f32", "f16", "local"),
+             ("f32", "bf16", "moment_sr")):
+    p = w.random_state_problem(61, 43, seed=3, bc=(0, 0, 1, 1), nonlinear=True, source="trig")
+    out = []
+    for variant in ("auto", "plain"):
+        lat = Lattice.from_problem(p, compute=form[0], storage=form[1], shift=form[2])
+        lat.set_sweep_variant(variant)
+        lat.init(p.phi0(), t0=p.t0).step(11).step(2)
+        assert lat.check() == 0 and lat.time()[0] == 13
+        out.append((lat.phi_host(), lat.read_f()))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+print("equal")
+"""
+
+
+def test_refused_cooperative_launch(tmp_path):
+    """A context with fewer SMs than the device (an MPS share, a green context) refuses the launch:
+    the lattice then advances in the other forms, bitwise the same."""
+    cc = shutil.which("gcc")
+    if cc is None:
+        pytest.skip("no gcc")
+    (tmp_path / "fake.c").write_text(FAKE)
+    so = tmp_path / "fake.so"
+    subprocess.run([cc, "-shared", "-fPIC", str(tmp_path / "fake.c"), "-o", str(so)], check=True)
+    r = subprocess.run([sys.executable, "-c", RUN % (ROOT, os.path.join(ROOT, "tests"))], capture_output=True, text=True,
+                       env=dict(os.environ, LD_PRELOAD=str(so)), timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert "equal" in r.stdout and r.stderr.count("refused") >= 5
