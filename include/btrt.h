@@ -209,8 +209,14 @@ btrt_status btrt_mass(btrt_lattice L, double *out);
 /* Flags raised by the sweep since the last btrt_init_phi: bit 0 = some node
  * produced a NaN/Inf phi (returns BTRT_EUNSTABLE), bit 2 = a bounded wait for a
  * tile copy or at a grid barrier gave up (returns BTRT_ETIMEOUT), bit 3 = an index check of a
- * -DBTRT_DEBUG_BOUNDS build failed (returns BTRT_ECUDA).  Synchronises. */
+ * -DBTRT_DEBUG_BOUNDS build failed (returns BTRT_ECUDA).  After a wait that gave up the
+ * state is undefined, although the step count went on, until btrt_init_phi or
+ * btrt_load sets it anew.  Synchronises. */
 btrt_status btrt_check(btrt_lattice L, int32_t *flags);
+
+/* Polls of a grid barrier (many steps per launch) before it gives up (default 2^22, some
+ * seconds). */
+btrt_status btrt_set_wait_limit(btrt_lattice L, uint64_t polls);
 
 /* Kernel form of the ordinary FP32-compute sweep: BTRT_SWEEP_AUTO (default: small
  * lattices advance up to 256 steps in one cooperative launch, in every format; the

@@ -96,6 +96,7 @@ SIGNATURES = [
     ("btrt_mass", ctypes.c_int, [_vp, _dp]),
     ("btrt_check", ctypes.c_int, [_vp, ctypes.POINTER(_i32)]),
     ("btrt_set_sweep_variant", ctypes.c_int, [_vp, _i32]),
+    ("btrt_set_wait_limit", ctypes.c_int, [_vp, ctypes.c_uint64]),
     ("btrt_auto_form", ctypes.c_int, [ctypes.POINTER(GridDesc), _i32, ctypes.POINTER(_i32)]),
     ("btrt_get_time", ctypes.c_int, [_vp, ctypes.POINTER(_i64), _dp]),
     ("btrt_state_bytes", _sz, [_vp]),

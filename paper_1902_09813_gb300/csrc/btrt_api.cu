@@ -513,7 +513,7 @@ btrt_status launch_tbn(btrt_lattice L, int n, bool *taken) {
     st.n = n;
     st.step0 = L->step + 1;
     st.barrier = L->barrier();
-    st.wait_limit = 1ull << 22;
+    st.wait_limit = L->wait_limit;
     for (int k = 0; k < n; ++k) {
         double sv = 0.0, wf = 1.0;
         step_scalars(L, L->step + 1 + k, false, &sv, &wf);
@@ -1070,6 +1070,12 @@ btrt_status btrt_set_sweep_variant(btrt_lattice L, int32_t variant) {
     if (variant == BTRT_SWEEP_TMA && !L->have_tma)
         return fail(BTRT_EINVAL, "the TMA sweep serves FP32-compute lattices whose tensor maps could be encoded");
     L->sweep_variant = variant;
+    return BTRT_OK;
+}
+
+btrt_status btrt_set_wait_limit(btrt_lattice L, uint64_t polls) {
+    if (!L) return fail(BTRT_EINVAL, "null lattice");
+    L->wait_limit = polls;
     return BTRT_OK;
 }
 

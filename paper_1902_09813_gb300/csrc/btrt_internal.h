@@ -67,6 +67,9 @@ struct btrt_lattice_s {
     CUtensorMap tma_out[2];
     bool have_tma = false;
     int sweep_variant = 0;    // BTRT_SWEEP_AUTO / PLAIN / TMA
+    // polls of a grid barrier (many steps per launch) before it gives up: some seconds, where a round
+    // takes some microseconds
+    unsigned long long wait_limit = 1ull << 22;
     bool have_srcf = false, have_af = false;   // fields uploaded
 
     // phi plane k; phi<Real>() is the current one (written with the populations of buffer cur)

@@ -196,6 +196,11 @@ class Lattice:
         C.check(self.lib.btrt_set_sweep_variant(self.handle, code))
         return self
 
+    def set_wait_limit(self, polls: int):
+        """Polls of a grid barrier (many steps per launch) before it gives up."""
+        C.check(self.lib.btrt_set_wait_limit(self.handle, int(polls)))
+        return self
+
     def set_coeffs(self, coef: C.Coeffs):
         self.coef = coef
         C.check(self.lib.btrt_set_coeffs(self.handle, ctypes.byref(coef)))
@@ -278,7 +283,7 @@ class Lattice:
         return flags.value
 
     def flags(self) -> int:
-        """The device flags without raising (bit 0: non-finite phi, bit 2: a tile-copy wait gave up)."""
+        """The device flags without raising (bit 0: non-finite phi, bit 2: a bounded wait gave up)."""
         flags = ctypes.c_int32()
         self.lib.btrt_check(self.handle, ctypes.byref(flags))
         return flags.value

@@ -1,11 +1,13 @@
-"""Many steps per launch: what its cooperative launch does when it is refused."""
+"""Many steps per launch: a refused cooperative launch, and a grid barrier that gives up."""
 import os
 import shutil
 import subprocess
 import sys
 
+import numpy as np
 import pytest
 
+import workloads as w
 from conftest import ROOT
 
 pytestmark = pytest.mark.gpu
@@ -53,3 +55,24 @@ def test_refused_cooperative_launch(tmp_path):
                        env=dict(os.environ, LD_PRELOAD=str(so)), timeout=600)
     assert r.returncode == 0, r.stderr[-2000:]
     assert "equal" in r.stdout and r.stderr.count("refused") >= 5
+
+
+@pytest.mark.parametrize("form", [("f64", "f64", "ref"), ("f32", "f32", "ref"), ("f32", "f16", "local")], ids="-".join)
+def test_barrier_that_gives_up(form):
+    """Blocks that find the others not yet there and may not wait: the launch ends, the check
+    says so, and a new initial field makes the lattice usable again."""
+    from paper_1902_09813_gb300 import Lattice
+    from paper_1902_09813_gb300 import _capi as C
+    p = w.random_state_problem(120, 90, seed=7, nonlinear=False, source="trig")
+    lat, ref = (Lattice.from_problem(p, compute=form[0], storage=form[1], shift=form[2]) for _ in range(2))
+    lat.set_wait_limit(0)
+    lat.init(p.phi0(), t0=p.t0).step(64)
+    with pytest.raises(C.BtrtError) as err:
+        lat.check()
+    assert err.value.code == C.ETIMEOUT and lat.flags() & 4
+    lat.set_wait_limit(1 << 22)
+    lat.init(p.phi0(), t0=p.t0).step(64)
+    ref.set_sweep_variant("plain")
+    ref.init(p.phi0(), t0=p.t0).step(64)
+    assert lat.check() == 0
+    assert np.array_equal(lat.phi_host(), ref.phi_host()) and np.array_equal(lat.read_f(), ref.read_f())
