@@ -76,3 +76,29 @@ def test_barrier_that_gives_up(form):
     ref.init(p.phi0(), t0=p.t0).step(64)
     assert lat.check() == 0
     assert np.array_equal(lat.phi_host(), ref.phi_host()) and np.array_equal(lat.read_f(), ref.read_f())
+
+
+@pytest.mark.parametrize("size,form,nonlinear", [
+    ((181, 181), ("f64", "f64", "ref"), False), ((131, 187), ("f64", "f64", "ref"), True),
+    ((255, 257), ("df64", "df64", "ref"), False), ((181, 181), ("df64", "df64", "ref"), True),
+    ((363, 361), ("f32", "f32", "ref"), True), ((33, 3971), ("f32", "f32", "local"), False),
+    ((511, 513), ("f32", "f16", "local"), True), ((8191, 32), ("f32", "bf16", "ref"), False),
+    ((511, 513), ("f32", "bf16", "moment_sr"), False), ((509, 515), ("f32", "f16", "local_sr"), True),
+    ((100, 2621), ("f32", "f16", "moment_sr"), True), ((511, 513), ("f32", "bf16", "local_dw_sr"), True),
+    ((49, 33), ("df64", "df64", "ref"), False), ((32, 49), ("df64", "df64", "ref"), True)],
+    ids=lambda v: "-".join(map(str, v)) if isinstance(v, tuple) else ("nonlinear" if v else "linear"))
+def test_largest_sizes(size, form, nonlinear):
+    """The largest lattices of the rule, with ragged tiles and more tiles than are resident: equal to
+    one step per launch bit for bit, and the many-steps form is the one that runs."""
+    from paper_1902_09813_gb300 import Lattice
+    from paper_1902_09813_gb300.lattice import auto_form
+    p = w.random_state_problem(*size, seed=12, bc=(0, 0, 1, 1), nonlinear=nonlinear, source="trig")
+    out = []
+    for variant in ("auto", "plain"):
+        lat = Lattice.from_problem(p, compute=form[0], storage=form[1], shift=form[2])
+        assert auto_form(lat.desc, nonlinear) == "many"
+        lat.set_sweep_variant(variant)
+        lat.init(p.phi0(), t0=p.t0).step(11)
+        assert lat.check() == 0
+        out.append((lat.phi_host(), lat.read_f()))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
