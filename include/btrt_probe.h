@@ -32,6 +32,10 @@ enum { BTRT_PROBE_FMA = 0, BTRT_PROBE_ADD = 1, BTRT_PROBE_MUL = 2 };
 btrt_status btrt_probe_fp64_rate(void *cuda_stream, int32_t kind, int32_t chains, int64_t iters, void *dev_sink,
                                  double *ops_per_s, double *ms);
 
+/* dev_out[i] = 1 / dev_v[i] by the reciprocal of the FP64 sweeps (n device values each; the
+ * call is asynchronous on cuda_stream).  BTRT_EINVAL for null arguments, n < 0 or above 2^31. */
+btrt_status btrt_probe_recip(void *cuda_stream, const double *dev_v, double *dev_out, int64_t n);
+
 #ifdef __cplusplus
 }
 #endif

@@ -122,6 +122,7 @@ SIGNATURES = [
     ("btrt_batch_destroy", ctypes.c_int, [_vp]),
     ("btrt_phi_sum_static", ctypes.c_int, [_vp, _i32, _i32, _i32, _i64, _vp, _dp]),
     ("btrt_probe_fp64_rate", ctypes.c_int, [_vp, _i32, _i32, _i64, _vp, _dp, _dp]),
+    ("btrt_probe_recip", ctypes.c_int, [_vp, _vp, _vp, _i64]),
     ("btrt3_workspace_bytes", _sz, [ctypes.POINTER(GridDesc3)]),
     ("btrt3_create", ctypes.c_int, [ctypes.POINTER(GridDesc3), _vp, _sz, _vp, ctypes.POINTER(_vp)]),
     ("btrt3_set_coeffs", ctypes.c_int, [_vp, ctypes.POINTER(Coeffs3)]),

@@ -37,6 +37,11 @@ __global__ void __launch_bounds__(kProbeThreads) fp64_chains(long long iters, do
     if (s == never) *sink = s;
 }
 
+__global__ void __launch_bounds__(kProbeThreads) recip_kernel(const double *v, double *out, long long n) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = btrt::recip_f64(v[i]);
+}
+
 template <int KIND, int CHAINS>
 cudaError_t time_chains(cudaStream_t s, long long iters, double *sink, double *ops_per_s, double *ms) {
     int dev = 0, sms = 0, per_sm = 0;
@@ -105,5 +110,21 @@ extern "C" btrt_status btrt_probe_fp64_rate(void *cuda_stream, int32_t kind, int
         return BTRT_ECUDA;
     }
     if (ms) *ms = t;
+    return BTRT_OK;
+}
+
+extern "C" btrt_status btrt_probe_recip(void *cuda_stream, const double *dev_v, double *dev_out, int64_t n) {
+    if (!dev_v || !dev_out || n < 0 || n > (1ll << 31)) {
+        btrt::set_last_error("btrt_probe_recip: null argument or count out of range");
+        return BTRT_EINVAL;
+    }
+    if (n == 0) return BTRT_OK;
+    recip_kernel<<<(unsigned)((n + kProbeThreads - 1) / kProbeThreads), kProbeThreads, 0,
+                   static_cast<cudaStream_t>(cuda_stream)>>>(dev_v, dev_out, n);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        btrt::set_last_error("btrt_probe_recip: %s", cudaGetErrorString(e));
+        return BTRT_ECUDA;
+    }
     return BTRT_OK;
 }
