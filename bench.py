@@ -75,14 +75,14 @@ def _header_count(name: str) -> int:
 # FP64 operations (add, mul or fma, one each) per node of the FP64 headline sweep's
 # scheme, counted from the kernel source next to collide_fold, in total and by kind.
 # The sweep runs most of them as 64-bit integer arithmetic (btrt_fx.cuh), so their
-# rate is not bounded by the FP64 pipe; its own bound is HBM (`hbm_view`).
+# rate is not bounded by the FP64 pipe; its own bound is HBM (binding_roofline).
 FP64_OPS_PER_UPDATE_LINEAR = _header_count("kFp64OpsPerNodeLinearTrig")
 FP64_MIX_PER_UPDATE = {"add": _header_count("kFp64AddsPerNodeLinearTrig"),
                        "fma": _header_count("kFp64FmasPerNodeLinearTrig"),
                        "mul": _header_count("kFp64MulsPerNodeLinearTrig")}
 # GB300's nominal FP64 rate, 1.25 TFLOP/s = 0.625 T FMA/s = 0.625 T FP64
 # operations/s when every add, mul or fma takes one lane slot; reported beside the
-# rate measured in the run (btrt_probe_fp64_rate), which is the roofline's peak.
+# rate measured in the run (btrt_probe_fp64_rate).
 FP64_NOMINAL_TOPS = 0.625
 # DRAM bytes per node of one FP64 sweep launch measured by ncu
 # (dram__bytes_read.sum + dram__bytes_write.sum) on the same kernel at 2048^2,
@@ -135,37 +135,30 @@ def measure_fp64_peak(iters: int = 2000):
             "kernel": "fp64_chains (4/8/16 independent chains per thread, whole waves, best per kind)"}
 
 
-def many_steps_form(args) -> bool:
-    """Small lattices: many steps per launch (the library's takes_tbn)."""
-    general = args.workload != "mms"
-    most = {"f64": 3 << 13 if general else 1 << 15, "df64": 1 << 15 if general else 1 << 16}.get(
-        args.compute, 1 << 17 if args.storage == "f32" and args.shift not in ("local_dw", "local_dw_sr") else 1 << 18)
-    return 32 <= args.n and args.n * args.n <= most
-
-
 def kernel_form(args) -> str:
-    """The kernel form of the timed steps: what the library's AUTO resolves to for
-    FP32 compute (the vector form for FP16/BF16 storage on lattices of 2^21 nodes
-    or more, two steps per launch otherwise), the form asked for, or the plain
-    sweep."""
-    if args.sweep == "auto" and many_steps_form(args):
-        return "tbn"
-    if args.compute != "f32" or args.shift in ("local_dw", "local_dw_sr"):
-        return "plain"
+    """The kernel form of the timed steps: the one asked for, or what the library's AUTO
+    takes on such a lattice ("many": many steps per launch)."""
     if args.sweep != "auto":
-        return args.sweep
-    large = args.n * args.n >= 1 << 21
-    if args.shift in ("local_sr", "moment_sr"):
-        large = large or (args.shift == "moment_sr" and args.storage == "bf16" and args.workload == "mms"
-                          and args.n * args.n >= 7 << 17)
-        return "vec" if large else "plain"
-    return "vec" if args.storage in ("f16", "bf16") and large else "tb2"
+        return args.sweep if args.compute == "f32" and args.shift not in ("local_dw", "local_dw_sr") else "plain"
+    import paper_1902_09813_gb300 as pkg
+    from paper_1902_09813_gb300.lattice import auto_form, grid_desc
+    pkg.build()
+    shift = args.shift if args.shift != "auto" else ("local" if args.storage in ("f16", "bf16") else "ref")
+    return auto_form(grid_desc(args.n, args.n, 1.0, 1.0, compute=args.compute, storage=args.storage, shift=shift),
+                     args.workload != "mms")
+
+
+def launches(args) -> int:
+    """Launches of the timed steps (many steps per launch: up to 256 in one)."""
+    form = kernel_form(args)
+    if form == "many":
+        return -(-args.steps // 256)
+    return args.steps // 2 + args.steps % 2 if two_step_form(args) else args.steps
 
 
 def two_step_form(args) -> bool:
     """Pairs of steps in one launch (the scalar or the vector two-step kernel)."""
     return kernel_form(args) in ("tb2", "tb2v")
-
 
 
 def roofline(args, nodes, t_launch, achieved_gbs, peak_hbm, peak_kind, fp64_peak=None):
@@ -186,6 +179,10 @@ def roofline(args, nodes, t_launch, achieved_gbs, peak_hbm, peak_kind, fp64_peak
         return dict(hbm, traffic=traffic, kernel=f"sweep_tb2_kernel<f32,{args.storage}>",
                     dram_bytes_per_update=per_update,
                     note="two steps per launch; achieved = algorithmic bytes of the steps / time")
+    if kernel_form(args) == "many":
+        # rounds of steps in shared memory over a state that L2 holds: no DRAM traffic to count
+        return dict(hbm, traffic=None, kernel=f"sweep_tbn_kernel<{args.compute},{args.storage}>",
+                    note="many steps per launch; achieved = algorithmic bytes of the steps / time")
     kernel = f"sweep_kernel<{args.compute},{args.storage}>"
     if kernel_form(args) == "vec":
         shift = args.shift if args.shift != "auto" else ("local" if args.storage in ("f16", "bf16") else "ref")
@@ -196,7 +193,7 @@ def roofline(args, nodes, t_launch, achieved_gbs, peak_hbm, peak_kind, fp64_peak
     if args.compute != "f64" or args.workload != "mms":
         return dict(hbm, traffic=None, kernel=kernel)
     # operations of the scheme against the FP64 pipe: above 1, since most of them run
-    # on the integer pipes; what bounds the sweep is HBM (hbm_view)
+    # on the integer pipes; what bounds the sweep is HBM (hbm_view, binding_roofline)
     tops = FP64_OPS_PER_UPDATE_LINEAR * nodes / t_launch / 1e12
     fresh = source_digest(FP64_SWEEP_SOURCES) == FP64_SWEEP_DIGEST
     traffic = round(FP64_TRAFFIC_PER_NODE * nodes) if fresh else None
@@ -213,6 +210,15 @@ def roofline(args, nodes, t_launch, achieved_gbs, peak_hbm, peak_kind, fp64_peak
             "note": "the scheme's FP64 operations; most run as 64-bit integer arithmetic, so the fraction "
                     "of the FP64 pipe exceeds 1 and hbm_view is the roofline that binds",
             "kernel": kernel, "hbm_view": hbm}
+
+
+def binding_roofline(r):
+    """The roofline that binds, for the JSON line: of the FP64 sweep HBM's, with its scheme's
+    operation rate beside it (11 of the 50 operations run on the FP64 pipe)."""
+    if "hbm_view" not in r:
+        return r
+    ops = {k: v for k, v in r.items() if k not in ("hbm_view", "traffic", "kernel")}
+    return dict(r["hbm_view"], traffic=r["traffic"], kernel=r["kernel"], fp64_scheme_view=ops)
 
 
 def _cores():
@@ -403,14 +409,13 @@ def run_gpu(args):
             "config": {"workload": desc, "nx": p.nx, "ny": p.ny,
                        "parallelism": "replicas" if ws > 1 else "single",
                        "l2": f"inputs {alg_bytes / 2 / 1e9:.2f} GB read per step >> L2, no flush"},
-            "roofline": roofline(args, nodes, t_launch, achieved_gbs, peak_hbm, peak_kind, fp64_peak),
+            "roofline": binding_roofline(roofline(args, nodes, t_launch, achieved_gbs, peak_hbm, peak_kind, fp64_peak)),
             "e2e": None if e2e_mlups is None else {
                 "value": round(e2e_mlups, 2), "unit": "MLUPS",
                 "h2d_bytes_per_step": int(8 * nodes / args.steps),
                 "d2h_bytes_per_step": int(8 * nodes / args.steps),
                 "note": "one solve per K steps: phi0 in, phi out, amortised per step"},
-            "gpu_launches": (args.steps // 2 + args.steps % 2) if two_step_form(args)
-            else -(-args.steps // 256) if kernel_form(args) == "tbn" else args.steps,
+            "gpu_launches": launches(args),
             "clocks": clk,
         }
         line.update(extra)
