@@ -332,7 +332,7 @@ __device__ __forceinline__ Real collide3(const Sweep3Params<Real> &p, Real (&d)[
 // ---------------------------------------------------------------- the FP64 collision on the integer pipes
 // As in two dimensions (btrt_fx.cuh, collide_f64): the FP64 forms out of line for
 // the nodes the integer form does not take.  FP64 alone takes 113 operations per node
-// and ran at 0.83 of the FP64 pipe, 4.3 GLUPS at 128^3; with the integer form 13.
+// and ran at 0.83 of the FP64 pipe, 4.3 GLUPS at 128^3; with the integer form 15.5.
 template <int MODE, int SRC>
 static __device__ __noinline__ double collide3_f64_slow(const Sweep3Params<double> &p, double *t, double phi_prev,
                                                         double srcv) {
@@ -464,9 +464,12 @@ BTRT_HD bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19],
     if constexpr (SRC != kSrcNone) src = p.src_val * srcv;
     if (SRC != kSrcNone && fx_exp(src) > em + (1u << 20)) return false;
     const bool k0_one = MODE == kLinearK0One || p.k0_one;
-    fx a, r[19];
-    if (k0_one) fx_density<true, SRC != kSrcNone, kFxTop3>(m.phi, FxArg{}, p.fx.om2, src, em, a);
-    else if (!fx_density<false, SRC != kSrcNone, kFxTop3>(m.phi, fx_arg(m.phi), p.fx.om2, src, em, a)) return false;
+    fx a = m.phi, r[19];
+    if (!k0_one) {
+        if (!fx_below3(m.phi)) return false;
+        a -= 2 * fx_mul(fx_arg(m.phi), p.fx.om2);
+    }
+    if (SRC != kSrcNone) a += fx_from<kFxTop3>(src, em);
     fx_expand3(a, z, X, Y, Z, fx_mul(fx_arg(m.hx), d12), fx_mul(fx_arg(m.hy), d12), fx_mul(fx_arg(m.t3), d24),
                fx_mul(fx_arg(m.pxy), d4), fx_mul(fx_arg(m.pxz), d4), fx_mul(fx_arg(m.pyz), d4), r);
     if (k0_one) fx_store<true, 0, kFxTop3>(D, r, p.fx.om2, em, d);

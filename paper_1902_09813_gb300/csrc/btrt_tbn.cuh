@@ -151,8 +151,6 @@ __device__ __forceinline__ void tbn_pull(const SweepParams<Real> &p, Real wall_f
     }
 }
 
-// st.n steps: p holds the parameters of the first (its inputs in fin, phi_in; the
-// other buffers in fout, phi_out; the rounds swap them).
 // Threads and resident blocks per SM the kernel is compiled for.  FP32 compute: two
 // blocks of 512 (64 registers), so that four of 256 fit as well: us per step at 256^2,
 // FP32 storage, manufactured solution / nonlinear 2.45 / 2.35 against 4.03 / 3.97 with the
@@ -164,6 +162,8 @@ template <typename Real, int MODE> struct TbnBounds {
     static constexpr int blocks = std::is_same<Real, dw>::value && MODE != kGeneral ? 3 : 2;
 };
 
+// st.n steps: p holds the parameters of the first (its inputs in fin, phi_in; the
+// other buffers in fout, phi_out; the rounds swap them).
 template <typename Real, typename S, int SH, int MODE, int SRC>
 __global__ void __launch_bounds__(TbnBounds<Real, MODE>::threads, TbnBounds<Real, MODE>::blocks)
     sweep_tbn_kernel(const __grid_constant__ SweepParams<Real> p, const __grid_constant__ TbnSteps<Real> st) {
