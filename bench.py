@@ -10,7 +10,8 @@ flush is needed between steps.
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
 Under torchrun (N > 1) every rank runs an independent replica (the method has
-no exchange between independent solves); rank 0 prints the JSON line.
+no exchange between independent solves); rank 0 prints the JSON line.  The whole
+tables of variants, accuracy and serving go to stderr as "bench details: {...}".
 """
 from __future__ import annotations
 
@@ -419,9 +420,41 @@ def run_gpu(args):
             "clocks": clk,
         }
         line.update(extra)
-        print(json.dumps(line), flush=True)
+        short, details = split_line(line)
+        if details:
+            print("bench details: " + json.dumps(details), file=sys.stderr, flush=True)
+        print(json.dumps(short), flush=True)
     if ws > 1:
         dist.destroy_process_group()
+
+
+# The variants that the line itself carries: the default form of each format.
+LINE_VARIANTS = ("mms_df64", "mms_f32_f32_tb2", "mms_f32_f16_local_vec", "mms_f32_bf16_moment_sr_vec", "nonlinear_f64",
+                 "nonlinear_f32_f32_tb2", "nonlinear_f32_f16_local_vec", "nonlinear_f32_bf16_moment_sr_vec",
+                 "d3q19_384_f64", "d3q19_384_f32_f32", "d3q19_384_f32_f16_local")
+
+
+def split_line(line):
+    """The JSON line and what goes to stderr beside it: the whole tables of variants, accuracy and
+    serving made the line some 20 KB long, which a reader that keeps the end of a log loses."""
+    short, details = dict(line), {}
+    if "variants" in line:
+        details["variants"] = line["variants"]
+        short["variants_mlups"] = {k: round(line["variants"][k]["mlups"]) for k in LINE_VARIANTS if k in line["variants"]}
+        del short["variants"]
+    if "accuracy" in line:
+        details["accuracy"] = line["accuracy"]
+        rel = line["accuracy"].get("nonlinear_8192_1000_rel_l2", {})
+        short["accuracy"] = {"nonlinear_8192_1000_rel_l2": {k: rel[k] for k in
+                             ("df64", "f32_f32_ref", "f32_f16_local", "f32_bf16_moment_sr") if k in rel}}
+    if "serving" in line:
+        details["serving"] = sv = line["serving"]
+        keys = ("solves_per_s", "p50_s", "p99_s", "gpu_idle_fraction")
+        short["serving"] = dict({k: v for k, v in sv.items() if not isinstance(v, dict)},
+                                rates={r: {k: v[k] for k in keys if k in v} for r, v in sv.get("rates", {}).items()},
+                                sequential_plain={k: v for k, v in sv.get("sequential_plain", {}).items() if k in keys},
+                                served_vs_sequential=sv.get("served_vs_sequential"))
+    return short, details
 
 
 # ---------------------------------------------------------------------------- variants

@@ -1,6 +1,7 @@
 """bench.py's kernel forms follow the library's choice, and its JSON line reports the
 roofline that binds."""
 import argparse
+import json
 
 import bench
 import pytest
@@ -40,3 +41,26 @@ def test_fp64_line_reports_hbm():
     assert r["bound"] == "hbm" and r["unit"] == "GB/s" and r["frac"] < 1.0
     assert r["traffic"] == round(bench.FP64_TRAFFIC_PER_NODE * nodes) and r["kernel"].startswith("sweep_kernel")
     assert r["fp64_scheme_view"]["ops_per_update"] == bench.FP64_OPS_PER_UPDATE_LINEAR
+
+
+def test_line_stays_short():
+    """The tables of a full run go beside the line, which keeps every contract key."""
+    contract = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline", "batched")
+    line = {k: {"filler": "x" * 120} for k in contract}
+    line["variants"] = {f"variant_{k}": {"mlups": 1e5, "ms_per_step": 0.5, "algorithmic_gbs": 6e3, "hbm_frac": 0.9}
+                        for k in range(70)}
+    line["variants"].update({k: {"mlups": 123456.7} for k in bench.LINE_VARIANTS})
+    line["accuracy"] = {t: {f"form_{k}": 1e-5 for k in range(16)} for t in
+                        ("nonlinear_2048_1000_rel_l2", "nonlinear_8192_1000_rel_l2", "hill_64_gre", "mms_128_gre")}
+    rate = {"solves_per_s": 29.2, "p50_s": 2.4, "p99_s": 2.6, "gpu_idle_fraction": 0.03,
+            "depth_t_active_waiting": [[0.1 * k, k, 96 - k] for k in range(40)]}
+    line["serving"] = {"requests_per_rate": 96, "rates": {r: rate for r in ("100", "500", "2000")},
+                       "sequential_plain": dict(rate), "served_vs_sequential": {"bitwise_equal": 96}}
+    short, details = bench.split_line(line)
+    assert len(json.dumps(line)) > 12000 and len(json.dumps(short)) < 6000
+    assert all(short[k] == line[k] for k in contract)
+    assert details == {k: line[k] for k in ("variants", "accuracy", "serving")}
+    assert short["variants_mlups"]["mms_df64"] == 123457 and short["serving"]["rates"]["500"]["p99_s"] == 2.6
+    plain, nothing = bench.split_line({k: line[k] for k in contract})
+    assert not nothing and plain == {k: line[k] for k in contract}
