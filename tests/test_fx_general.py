@@ -215,6 +215,35 @@ def test_errors_no_larger_than_plain_fp64(lib, dim, k0):
     assert (e[0] <= e[1]).all(), np.sqrt(e / n)
 
 
+@pytest.mark.parametrize("k0", [1.0, 0.05, 1.4, 1.7, 1.89, 1.98])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_ends_of_the_word(lib, dim, k0):
+    """Populations at the top of a binade, one sign or signs that add up along a direction: right to
+    16 roundings of the largest of the sums (20 populations), or refused and untouched."""
+    rng = np.random.default_rng(int(100 * k0))
+    Q, taken = len(VEL[dim]), 0
+    for _ in range(300):
+        k2, um, rate = rng.choice([-1.0, 0.02, 0.7, 1.98]), rng.choice([0.05, 0.49, 0.7, 0.99]), rng.choice([0.0, 0.05])
+        c = _coeffs(rng, dim, 2.0, rng.choice([0.0, 0.05]), k0, k2, rate, um)
+        c[-1] = 2.0
+        if rng.random() < 0.3:                              # K1 near 2
+            c[2 * dim + 2:-5] = [1e-4 if a == b else 0.0 for a in range(dim) for b in range(a, dim)]
+        towards = VEL[dim][rng.integers(0, Q)]
+        s = [np.ones(Q), rng.choice([-1.0, 1.0], size=Q), rng.uniform(-1.0, 1.0, size=Q),
+             np.array([1.0 if np.dot(towards, v) >= 0 else -1.0 for v in VEL[dim]])][rng.integers(0, 4)]
+        top = 0.25 * (2.0 - 2.0 ** -52)
+        d, prev = list(rng.choice([-1.0, 1.0]) * top * s), rng.uniform(-4.0, 4.0) * top
+        ok, got, phi = _node(lib, c, d, prev)
+        taken += ok == 1
+        if ok != 1:
+            assert got == d
+            continue
+        ref, rphi, _ = _collide(c, d, prev, Decimal, dim)
+        for g, r in zip(got + [phi], ref + [rphi]):
+            assert abs(Decimal(g) - r) <= 16 * 20 * Decimal(2) ** -53 * Decimal(top)
+    assert taken > 20
+
+
 @pytest.mark.parametrize("k2", [-1.0, 0.7])
 @pytest.mark.parametrize("dim", [2, 3])
 def test_coefficients_past_the_reciprocal(lib, dim, k2):
