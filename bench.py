@@ -92,7 +92,7 @@ FP64_NOMINAL_TOPS = 0.625
 # to them both are re-taken and the digest updated (a CPU test checks it), and
 # until then the traffic is reported as null.
 FP64_SWEEP_SOURCES = ("btrt_sweep.cuh", "btrt_dw.cuh", "btrt_fx.cuh")   # the FP64 sweep's device code
-FP64_SWEEP_DIGEST = "f48db7915d685688"
+FP64_SWEEP_DIGEST = "d1ddad3a0363a873"
 FP64_TRAFFIC_PER_NODE = 148.1
 # DRAM bytes per node and step of the two-step FP32-compute kernel measured by ncu,
 # keyed by (storage, shift), for the sources with digest TB2_DIGEST.

@@ -193,12 +193,11 @@ struct FxFold {
     FxConst Qxx, Qxy, Qyy, Px, Py, gx, gy, d18, d4, om2;
     FxConst ux, uy, k06;   // per-node coefficients: u^ and k0/6
     int ok;          // kFxOk* bits; a form whose bit is not set takes the FP64 collision
-    short hx, hy;    // kFxHalves: u^ is h/2 more than its constant
+    int ush;         // u^ is its constant times 2^ush
     double trh, detA;      // half the trace and the determinant of A0^
 };
-// om2, u^ and k0/6 fit; the constant-coefficient form's fit; bgx = bgy; c3 != 0; a
-// component of u^ is a half or more
-enum { kFxOkGeneral = 1, kFxOkLinear = 2, kFxSameB = 4, kFxC3 = 8, kFxHalves = 16 };
+// om2, u^ and k0/6 fit; the constant-coefficient form's fit; bgx = bgy; c3 != 0
+enum { kFxOkGeneral = 1, kFxOkLinear = 2, kFxSameB = 4, kFxC3 = 8 };
 
 // A constant as the products see it.
 inline double fx_real(const FxConst &c) { return ldexp((double)c.hi, -32) + ldexp((double)c.lo, -64); }
@@ -243,11 +242,10 @@ inline bool fx_linear_fits(const FxFold &q) {
 // = 8.3, since K1's eigenvalues lie in (0, 2) and E is tested against 4.
 inline FxFold fx_fold(const double (&Q)[3], const double (&P)[2], const double (&g)[2], double dk, double om,
                       const double (&u)[2], double k0) {
-    // a constant holds less than a half: from there on u^ is split into h/2 and a rest
-    const auto half = [](double t) { return t >= 0.4999 ? 1 : t <= -0.4999 ? -1 : 0; };
-    const int hx = half(u[0]), hy = half(u[1]);
-    const double v[13] = {-Q[0], -Q[1], -Q[2], P[0],           P[1],           -g[0], -g[1],
-                          dk,    dk,    om,    u[0] - 0.5 * hx, u[1] - 0.5 * hy, k0};
+    // a constant holds less than a half: from there on it is half of u^, and the product doubled
+    const int ush = fabs(u[0]) >= 0.4999 || fabs(u[1]) >= 0.4999 ? 1 : 0;
+    const double us = ush ? 0.5 : 1.0;
+    const double v[13] = {-Q[0], -Q[1], -Q[2], P[0], P[1], -g[0], -g[1], dk, dk, om, us * u[0], us * u[1], k0};
     const int div[13] = {6, 6, 6, 6, 6, 6, 6, 18, 4, 2, 1, 1, 6};
     FxConst k[13];
     bool fit[13], lin = true;
@@ -256,17 +254,22 @@ inline FxFold fx_fold(const double (&Q)[3], const double (&P)[2], const double (
         k[i] = fx_const(fit[i] ? v[i] : 0.0, div[i]);
         if (i < 10) lin = lin && fit[i];
     }
-    FxFold q = {k[0], k[1], k[2], k[3], k[4], k[5], k[6], k[7], k[8], k[9], k[10], k[11], k[12], 0, (short)hx, (short)hy, 0.0, 0.0};
+    FxFold q = {k[0], k[1], k[2], k[3], k[4], k[5], k[6], k[7], k[8], k[9], k[10], k[11], k[12], 0, ush, 0.0, 0.0};
     lin = lin && fx_flux_fits(q.Qxx, q.Qxy, q.Px, q.gx) && fx_flux_fits(q.Qxy, q.Qyy, q.Py, q.gy) && fx_linear_fits(q);
     // the low products of k0 j/6 + B's change/6 (up to 15 units) sum below 2^63 up to k0 = 1.9
-    const bool halves = hx || hy, gen = fit[9] && fit[10] && fit[11] && fit[12] && (!halves || k0 < 1.9);
-    q.ok = (gen ? kFxOkGeneral : 0) | (lin ? kFxOkLinear : 0) | (halves ? kFxHalves : 0);
+    const bool gen = fit[9] && fit[10] && fit[11] && fit[12] && (!ush || k0 < 1.9);
+    q.ok = (gen ? kFxOkGeneral : 0) | (lin ? kFxOkLinear : 0);
     return q;
 }
 
 // Sums whose terms may pass 2^63 (the caller tests the result before it is used).
 BTRT_HD fx fx_plus(fx a, fx b) { return (fx)((unsigned long long)a + (unsigned long long)b); }
 BTRT_HD fx fx_minus(fx a, fx b) { return (fx)((unsigned long long)a - (unsigned long long)b); }
+BTRT_HD fx fx_times2(fx a, int sh) { return (fx)((unsigned long long)a << sh); }   // a 2^sh
+// |phi| below LIMIT (in units of 2^32).
+template <int LIMIT> BTRT_HD bool fx_below(fx phi) {
+    return (unsigned int)((int)(phi >> 32) + LIMIT) < 2u * (unsigned int)LIMIT;
+}
 
 // a = k0 phi + source of a node; false when it could leave its word.  With k0 = 1 it
 // cannot (nine populations below 2^59 units and a source below 2^60; in three dimensions
@@ -338,22 +341,24 @@ template <int N> BTRT_HD bool fx_common_exp(const double (&d)[N], unsigned int &
 }
 
 // Whether a node is zero throughout (its results then are as well).
-BTRT_HD bool fx_all_zero(const double *d, int n, double phi_prev, double src) {
+template <int N> BTRT_HD bool fx_all_zero(const double (&d)[N], double phi_prev, double src) {
     unsigned long long any = fx_bits(phi_prev) | fx_bits(src);
-    for (int i = 0; i < n; ++i) any |= fx_bits(d[i]);
+#pragma unroll
+    for (int i = 0; i < N; ++i) any |= fx_bits(d[i]);
     return (any << 1) == 0;
 }
 // A node whose largest population is out of the range: large values take the FP64 form, and
 // so do tiny ones, for its gradual underflow; zeros are done.  On the device the
-// out-of-line FP64 forms look for those: with the test in line the 8192^2 sweep took
-// 38.56 ms instead of 37.48.
-template <int N> BTRT_HD bool fx_out_of_range(const double (&d)[N], double phi_prev, double src, double &phi_out) {
+// out-of-line FP64 forms of the one-step sweeps look for those: with the test in line the
+// 8192^2 sweep took 38.56 ms instead of 37.48.  ZEROS: in line all the same (many steps per
+// launch: the 64^2 hill 0.959 ms against 0.977).
+template <bool ZEROS, int N>
+BTRT_HD bool fx_out_of_range(const double (&d)[N], double phi_prev, double src, double &phi_out) {
 #ifdef __CUDA_ARCH__
-    return false;
-#else
-    phi_out = 0.0;
-    return fx_all_zero(d, N, phi_prev, src);
+    if (!ZEROS) return false;
 #endif
+    phi_out = 0.0;
+    return fx_all_zero(d, phi_prev, src);
 }
 
 // The outputs of a node, (1 - k0) D_i + r_i, as FP64; the first NADD by the FP64
@@ -380,11 +385,12 @@ BTRT_HD void fx_store(const fx (&D)[N], const fx (&r)[N], const FxConst &om2, un
 // d untouched, when the node's values leave the range (the caller takes the FP64
 // form): the exponents of the populations, or phi^{n-1} or the source more than four
 // times or twice the largest population.
-template <bool K0ONE, bool SOURCE>
+template <bool K0ONE, bool SOURCE, bool ZEROS = false>
 BTRT_HD bool fx_collide_linear(const FxFold &q, double (&d)[9], double phi_prev, double src, double &phi_out) {
     unsigned int em;
-    if (!fx_common_exp(d, em)) return fx_out_of_range(d, phi_prev, SOURCE ? src : 0.0, phi_out);
-    if (fx_exp(phi_prev) > em + (2u << 20)) return false;
+    const bool in = fx_common_exp(d, em);
+    if (!in || fx_exp(phi_prev) > em + (2u << 20))
+        return !in && fx_out_of_range<ZEROS>(d, phi_prev, SOURCE ? src : 0.0, phi_out);
     if (SOURCE && fx_exp(src) > em + (1u << 20)) return false;
     fx D[9];
 #pragma unroll
@@ -510,15 +516,6 @@ inline FxFold3 fx_fold3(const double (&Q)[6], const double (&P)[3], const double
     return q;
 }
 
-// |phi| below 15 2^58 units: k0 phi + source then stays in its word for every k0 below 2.  The
-// per-node form takes this test where k0 is not 1 (183 x 34 x 154, nonlinear, 14 steps: 2.89 ms
-// against 2.90 with fx_density's); nodes above it, of nineteen populations nearly as
-// large as the largest, are rare.
-BTRT_HD bool fx_below3(fx phi) {
-    constexpr int limit = 15 << 26;
-    return (unsigned int)((int)(phi >> 32) + limit) < 2u * (unsigned int)limit;
-}
-
 struct FxMoments3 {
     fx phi, jx, jy, jz, pxy, pxz, pyz;
     fx hx, hy, t3;   // 3 h_x, 3 h_y (h_z = -h_x - h_y) and 3 t3
@@ -586,8 +583,9 @@ BTRT_HD void fx_expand3(fx a, fx z, fx X, fx Y, fx Z, fx Hx, fx Hy, fx K, fx txy
 template <bool K0ONE, bool SOURCE>
 BTRT_HD bool fx_collide_linear3(const FxFold3 &q, double (&d)[19], double phi_prev, double src, double &phi_out) {
     unsigned int em;
-    if (!fx_common_exp(d, em)) return fx_out_of_range(d, phi_prev, SOURCE ? src : 0.0, phi_out);
-    if (fx_exp(phi_prev) > em + (2u << 20)) return false;
+    const bool in = fx_common_exp(d, em);
+    if (!in || fx_exp(phi_prev) > em + (2u << 20))
+        return !in && fx_out_of_range<false>(d, phi_prev, SOURCE ? src : 0.0, phi_out);
     if (SOURCE && fx_exp(src) > em + (1u << 20)) return false;
     fx D[19];
 #pragma unroll

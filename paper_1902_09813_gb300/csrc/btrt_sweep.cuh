@@ -477,7 +477,7 @@ __device__ __forceinline__ double collide_f64_plain(const SweepParams<double> &p
     double d[9], phid;
 #pragma unroll
     for (int i = 0; i < 9; ++i) d[i] = t[i];
-    if (fx_all_zero(d, 9, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv)) return 0.0;
+    if (fx_all_zero(d, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv)) return 0.0;
     const double phi =
         collide_fold<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, node, phid, nullptr, sv);
 #pragma unroll
@@ -515,20 +515,40 @@ BTRT_HD double recip_f64(double v) {
 // the nonlinear terms and K1 are FP64 (26 operations instead of 97; the two divisions
 // share one reciprocal).  Returns false, with d untouched, when a value leaves
 // the integer form's range.
-template <int MODE, int SRC>
+template <int MODE, int SRC, bool ZEROS = false>
 BTRT_HD bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], double phi_prev,
                                                    double srcv, int node, double src_val, double &phi_out) {
     const FoldConsts<double> &L = p.lin;
     unsigned int em;
-    if (!fx_common_exp(d, em)) return fx_out_of_range(d, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv, phi_out);
-    if (fx_exp(phi_prev) > em + (2u << 20)) return false;
+    const bool in = fx_common_exp(d, em);
+    if (!in || fx_exp(phi_prev) > em + (2u << 20))
+        return !in && fx_out_of_range<ZEROS>(d, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv, phi_out);
     fx D[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) D[i] = fx_from(d[i], em);
     FxMoments m = fx_moments(D);
     const double phi = fx_to(m.phi, em);
-    fx X, Y, z = 0;
+    fx X, Y, z = 0, a;
     FxConst d4, d18;
+    const bool k0_one = MODE == kLinearK0One || p.k0_one;
+    // a = k0 phi + source and whether it stays in its word.  Formed before the flux's test, which
+    // then covers both (late / early, ms: 900 x 900 per-node tensor 2.86 / 2.80, 128^2 nonlinear, 200 steps
+    // 1.885 / 1.855), but for a reaction source, whose powers would lengthen the way to that
+    // test (1024^2 front 7.79 / 7.86, 128^2 2.77 / 2.82).
+    constexpr bool EARLY = MODE == kGeneral && SRC != kSrcReaction && SRC != kSrcRuntime;
+    const auto density = [&]() {
+        double src = 0.0;
+        if constexpr (SRC == kSrcReaction || SRC == kSrcRuntime) {
+            if (SRC == kSrcReaction || p.src_kind == kSrcReaction)
+                srcv = fma(1.5, reaction(p, phi), -0.5 * reaction(p, phi_prev));
+        }
+        if constexpr (SRC != kSrcNone) src = src_val * srcv;
+        if (SRC != kSrcNone && fx_exp(src) > em + (1u << 20)) return false;
+        return k0_one ? fx_density<true, SRC != kSrcNone, 58>(m.phi, FxArg{}, p.fx.om2, src, em, a)
+                      : fx_density<false, SRC != kSrcNone, 58>(m.phi, fx_arg(m.phi), p.fx.om2, src, em, a);
+    };
+    bool fits = true;
+    if constexpr (EARLY) fits = density();
     if constexpr (MODE == kGeneral) {
         // V = K1 (B - dB/2 - j) + k0 j + dB with B = u phi + bg g(phi), g = phi^q: the linear
         // parts and j stay integers; g's mean (over phi, phi^{n-1}) and difference are FP64
@@ -552,15 +572,11 @@ BTRT_HD bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], do
         const unsigned int far = em + (1u << 20);
         if (fx_exp(gsx) > far || fx_exp(gsy) > far || fx_exp(gdx) > far || fx_exp(gdy) > far) return false;
         const FxArg mean = fx_arg((m.phi + pv) >> 1), diff = fx_arg(m.phi - pv);
-        fx Ex = fx_mul(mean, p.fx.ux) + fx_from(gsx, em) - m.jx, Ey = fx_mul(mean, p.fx.uy) + fx_from(gsy, em) - m.jy;
-        fx Dx = fx_mul(diff, p.fx.ux) + fx_from(gdx, em), Dy = fx_mul(diff, p.fx.uy) + fx_from(gdy, em);
-        if (p.fx.ok & kFxHalves) {   // u^ = h/2 and the constant (all FP64 instead: 846 us at 2048^2, not 265)
-            const fx mh = (m.phi + pv) >> 2, dh = (m.phi - pv) >> 1;
-            Ex += p.fx.hx * mh;
-            Ey += p.fx.hy * mh;
-            Dx += p.fx.hx * dh;
-            Dy += p.fx.hy * dh;
-        }
+        const int sh = p.fx.ush;
+        const fx Ex = fx_times2(fx_mul(mean, p.fx.ux), sh) + fx_from(gsx, em) - m.jx;
+        const fx Ey = fx_times2(fx_mul(mean, p.fx.uy), sh) + fx_from(gsy, em) - m.jy;
+        const fx Dx = fx_times2(fx_mul(diff, p.fx.ux), sh) + fx_from(gdx, em);
+        const fx Dy = fx_times2(fx_mul(diff, p.fx.uy), sh) + fx_from(gdy, em);
         const double p2 = phi * phi;
         if (p.fx.ok & kFxC3) {
             // C(phi) - phi: in sigma, and k0 (C - phi) / 18 in the isotropic terms
@@ -598,8 +614,7 @@ BTRT_HD bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], do
         if (fx_exp(Kxx) > (1021u << 20) || fx_exp(Kxy) > (1021u << 20) || fx_exp(Kyy) > (1021u << 20) ||
             fx_exp(dk) > (1023u << 20))
             return false;
-        if ((unsigned int)((int)(Ex >> 32) + (1 << 29)) >= (1u << 30) || (unsigned int)((int)(Ey >> 32) + (1 << 29)) >= (1u << 30))
-            return false;
+        if (!fx_below<1 << 29>(Ex) || !fx_below<1 << 29>(Ey) || !fits) return false;
         auto konst = [](double v, unsigned int one) {          // one: the exponent of the unit 2^-64
             const FxArg c = fx_arg(fx_from(v, one));
             return FxConst{c.h, c.l};
@@ -637,18 +652,11 @@ BTRT_HD bool fx_collide_general(const SweepParams<double> &p, double (&d)[9], do
         d4 = p.fx.d4;
         d18 = p.fx.d18;
     }
-    double src = 0.0;
-    if constexpr (SRC == kSrcReaction || SRC == kSrcRuntime) {
-        if (SRC == kSrcReaction || p.src_kind == kSrcReaction)
-            srcv = fma(1.5, reaction(p, phi), -0.5 * reaction(p, phi_prev));
+    if constexpr (!EARLY) {
+        if (!density()) return false;
     }
-    if constexpr (SRC != kSrcNone) src = src_val * srcv;
-    if (SRC != kSrcNone && fx_exp(src) > em + (1u << 20)) return false;
     const fx ks = fx_mul(fx_arg(m.s32), d18), t1 = fx_mul(fx_arg(m.del), d4), t5 = fx_mul(fx_arg(m.pxy), d4);
-    fx a, r[9];
-    const bool k0_one = MODE == kLinearK0One || p.k0_one;
-    if (k0_one) fx_density<true, SRC != kSrcNone, 58>(m.phi, FxArg{}, p.fx.om2, src, em, a);
-    else if (!fx_density<false, SRC != kSrcNone, 58>(m.phi, fx_arg(m.phi), p.fx.om2, src, em, a)) return false;
+    fx r[9];
     fx_expand(a, z, X, Y, ks, t1, t5, r);
     // the FP64 pipe bounds the per-node coefficients; the constant ones are converted as in
     // fx_collide_linear (ties round differently in the two conversions)
@@ -713,11 +721,11 @@ __device__ __forceinline__ double collide_f64(const SweepParams<double> &p, doub
     bool done = false;
     if (p.fx.ok & (MODE == kGeneral ? kFxOkGeneral : kFxOkLinear)) {
         if constexpr (MODE == kGeneral || LATE)
-            done = fx_collide_general<MODE, SRC>(p, d, phi_prev, srcv, node, src_val, phi);
+            done = fx_collide_general<MODE, SRC, OWN>(p, d, phi_prev, srcv, node, src_val, phi);
         else if (MODE == kLinearK0One || p.k0_one)
-            done = fx_collide_linear<true, SRC != kSrcNone>(p.fx, d, phi_prev, SRC != kSrcNone ? src_val * srcv : 0.0, phi);
+            done = fx_collide_linear<true, SRC != kSrcNone, OWN>(p.fx, d, phi_prev, SRC != kSrcNone ? src_val * srcv : 0.0, phi);
         else
-            done = fx_collide_linear<false, SRC != kSrcNone>(p.fx, d, phi_prev, SRC != kSrcNone ? src_val * srcv : 0.0, phi);
+            done = fx_collide_linear<false, SRC != kSrcNone, OWN>(p.fx, d, phi_prev, SRC != kSrcNone ? src_val * srcv : 0.0, phi);
     }
     if (!done) {
         double t[9];

@@ -339,7 +339,7 @@ static __device__ __noinline__ double collide3_f64_slow(const Sweep3Params<doubl
     double d[19], phid;
 #pragma unroll
     for (int i = 0; i < 19; ++i) d[i] = t[i];
-    if (fx_all_zero(d, 19, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv)) return 0.0;
+    if (fx_all_zero(d, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv)) return 0.0;
     const double phi = collide3<double, MODE, SRC, kShiftNone>(p, d, 0.0, phi_prev, srcv, false, phid);
 #pragma unroll
     for (int i = 0; i < 19; ++i) t[i] = d[i];
@@ -362,13 +362,16 @@ template <int MODE, int SRC>
 BTRT_HD bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19], double phi_prev,
                                                     double srcv, double &phi_out) {
     unsigned int em;
-    if (!fx_common_exp(d, em)) return fx_out_of_range(d, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv, phi_out);
-    if (fx_exp(phi_prev) > em + (2u << 20)) return false;
+    const bool in = fx_common_exp(d, em);
+    if (!in || fx_exp(phi_prev) > em + (2u << 20))
+        return !in && fx_out_of_range<false>(d, phi_prev, SRC == kSrcNone || SRC == kSrcReaction ? 0.0 : srcv, phi_out);
     fx D[19];
 #pragma unroll
     for (int i = 0; i < 19; ++i) D[i] = fx_from<kFxTop3>(d[i], em);
     FxMoments3 m = fx_moments3(D);
     const double phi = fx_to<kFxTop3>(m.phi, em);
+    // k0 phi + source stays in its word below 15 2^58 units for every k0 below 2
+    const bool k0_one = MODE == kLinearK0One || p.k0_one, fits = k0_one || fx_below<15 << 26>(m.phi);
     fx X, Y, Z, z = 0;
     FxConst d12, d24, d4;
     if constexpr (MODE == kGeneral) {
@@ -418,7 +421,6 @@ BTRT_HD bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19],
             id = recip_f64(det);
             k2 = p.k2c;
         }
-        if (fx_exp(id) == 0) return false;   // the reciprocal underflowed (and k2 with it)
         const double dk = k2 - p.k0;
         // K1 e with the cofactors, divided by the determinant once per component
         const double ex = id * fma(-0.5, dBx, Bx - jx), ey = id * fma(-0.5, dBy, By - jy), ez = id * fma(-0.5, dBz, Bz - jz);
@@ -426,7 +428,9 @@ BTRT_HD bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19],
         const double Vy = fma(cxy, ex, fma(cyy, ey, fma(cyz, ez, fma(p.k0, jy, dBy))));
         const double Vz = fma(cxz, ex, fma(cyz, ey, fma(czz, ez, fma(p.k0, jz, dBz))));
         const unsigned int far = em + (2u << 20);
-        if (fx_exp(dk) > (1023u << 20) || fx_exp(Vx) > far || fx_exp(Vy) > far || fx_exp(Vz) > far) return false;
+        // id 0: the reciprocal underflowed (and k2 with it)
+        if (fx_exp(dk) > (1023u << 20) || fx_exp(Vx) > far || fx_exp(Vy) > far || fx_exp(Vz) > far || fx_exp(id) == 0 || !fits)
+            return false;
         const FxConst sixth = {0x2aaaaaab, (int)0xaaaaaaab};   // 2^64 / 6
         X = fx_mul(fx_arg(fx_from<kFxTop3>(Vx, em)), sixth);
         Y = fx_mul(fx_arg(fx_from<kFxTop3>(Vy, em)), sixth);
@@ -463,12 +467,9 @@ BTRT_HD bool fx_collide_general3(const Sweep3Params<double> &p, double (&d)[19],
     if constexpr (SRC == kSrcReaction) srcv = fma(1.5, reaction3(p, phi), -0.5 * reaction3(p, phi_prev));
     if constexpr (SRC != kSrcNone) src = p.src_val * srcv;
     if (SRC != kSrcNone && fx_exp(src) > em + (1u << 20)) return false;
-    const bool k0_one = MODE == kLinearK0One || p.k0_one;
+    if (MODE != kGeneral && !fits) return false;
     fx a = m.phi, r[19];
-    if (!k0_one) {
-        if (!fx_below3(m.phi)) return false;
-        a -= 2 * fx_mul(fx_arg(m.phi), p.fx.om2);
-    }
+    if (!k0_one) a -= 2 * fx_mul(fx_arg(m.phi), p.fx.om2);
     if (SRC != kSrcNone) a += fx_from<kFxTop3>(src, em);
     fx_expand3(a, z, X, Y, Z, fx_mul(fx_arg(m.hx), d12), fx_mul(fx_arg(m.hy), d12), fx_mul(fx_arg(m.t3), d24),
                fx_mul(fx_arg(m.pxy), d4), fx_mul(fx_arg(m.pxz), d4), fx_mul(fx_arg(m.pyz), d4), r);
