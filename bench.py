@@ -93,17 +93,17 @@ FP64_NOMINAL_TOPS = 0.625
 # until then the traffic is reported as null.
 FP64_SWEEP_SOURCES = ("btrt_sweep.cuh", "btrt_dw.cuh", "btrt_fx.cuh")   # the FP64 sweep's device code
 FP64_SWEEP_DIGEST = "d1ddad3a0363a873"
-FP64_TRAFFIC_PER_NODE = 148.1
+FP64_TRAFFIC_PER_NODE = 148.2
 # DRAM bytes per node and step of the two-step FP32-compute kernel measured by ncu,
 # keyed by (storage, shift), for the sources with digest TB2_DIGEST.
 TB2_SOURCES = ("btrt_sweep.cuh", "btrt_tb.cuh", "btrt_launch.cuh")
-TB2_DIGEST = "31c45d2ca3d73372"
+TB2_DIGEST = "3aa83debfef4c501"
 TB2_DRAM_BYTES_PER_UPDATE = {("f32", "ref"): 38.7, ("f16", "local"): 20.9}
 # DRAM bytes per node of one launch of the vector-access sweep measured by ncu,
 # keyed by (storage, shift), for the sources with digest VEC_DIGEST.
 VEC_SOURCES = ("btrt_sweep.cuh", "btrt_vec.cuh", "btrt_launch.cuh")
-VEC_DIGEST = "54ee35884fdb823b"
-VEC_DRAM_BYTES_PER_UPDATE = {("f16", "local"): 41.3, ("f16", "local_sr"): 41.1}
+VEC_DIGEST = "1be18ff24b04780b"
+VEC_DRAM_BYTES_PER_UPDATE = {("f16", "local"): 41.4, ("f16", "local_sr"): 41.1}
 
 
 def measure_fp64_peak(iters: int = 2000):
